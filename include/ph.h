@@ -252,8 +252,11 @@ ph_status ph_recover_factored_dw(const ph_mesh* mesh, const double* factor, doub
  * preconditioner, starting from x = 0, until ||r||_2 <= rtol ||b||_2 or
  * maxit iterations.  x [n] float64 out.  iters / relres (host pointers, may
  * be NULL) receive the iteration count and the final relative residual.
- * Allocates 5n + O(1) doubles of workspace from the library's pool and
- * synchronises `stream` every 8 iterations to test convergence.
+ * Convergence is tested every 8 iterations.  Allocates 5n + O(1) doubles of
+ * workspace (and a copy of H where its rows hold at most 16 entries) from the
+ * library's pool and synchronises `stream` every 8 iterations, or for systems
+ * of at most 311,296 rows every 4096 (their test runs on the device, in one
+ * cooperative launch).  A device-side wait that runs out gives PH_ERR_TIMEOUT.
  * Errors: PH_ERR_NOT_CONVERGED when maxit is reached (x holds the last
  * iterate); PH_ERR_ARG for a non-positive diagonal entry.
  */
@@ -289,8 +292,7 @@ ph_status ph_solve_pcg(int64_t n, const int32_t* rowptr, const int32_t* colind, 
  *   from several streams or threads, race on it: serialise them.
  * Never calls cudaMalloc, cudaFree or any allocating routine.  Like
  * ph_solve_pcg, it copies the convergence test's scalars to the host and
- * waits for `stream` every 8 iterations, so it returns only when the solve is
- * done.
+ * waits for `stream`, so it returns only when the solve is done.
  */
 ph_status ph_solve_pcg_noalloc(int64_t n, const int32_t* rowptr, const int32_t* colind, const double* values,
                                const double* b, double* x, double rtol, int32_t maxit, int32_t* iters,

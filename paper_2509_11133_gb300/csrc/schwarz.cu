@@ -37,9 +37,6 @@ __device__ __forceinline__ void faces_of_edge(int j, int& a, int& b) {
   b = B[j];
 }
 
-// Position of (i, j), i <= j, in a packed row-major upper triangle of order k.
-__host__ __device__ __forceinline__ int upper(int i, int j, int k) { return i * k - i * (i - 1) / 2 + (j - i); }
-
 // Incidences per edge (faces with a multiplier, counted from their T+ tet)
 // and the edge's vertex pair (written by its first occurrence).
 __global__ void k_patch_count(const int4* __restrict__ tet, const int4* __restrict__ tface,
@@ -145,13 +142,6 @@ __device__ __forceinline__ double csr_entry(const int32_t* __restrict__ rowptr, 
   return 0.0;
 }
 
-// Group of patch index t (patches ordered by group).
-__device__ __forceinline__ int group_of(const SchwarzGroups& g, int64_t t) {
-  int k = 1;
-  while (k < kSchwarzDense && t >= g.first[k + 1]) ++k;
-  return k;
-}
-
 // Invert each patch block: Cholesky A = G G', then A^-1 = G^-T G^-1 (upper
 // triangle stored, slot-major within the group).
 __global__ void k_group_factor(SchwarzGroups g, int64_t npatch, const int32_t* __restrict__ mem,
@@ -205,58 +195,13 @@ __global__ void k_mult_to_face(const int32_t* __restrict__ face_mult, int64_t nF
   if (F < nF && face_mult[F] >= 0) m2f[face_mult[F]] = (int)F;
 }
 
-// y = block^-1 r_patch for one patch of K members (slot-major group arrays,
-// stride n): the packed inverse in registers, sums in member order.
-template <int K>
-__device__ __forceinline__ void patch_solve(int64_t s, int64_t n, const int32_t* __restrict__ mem,
-                                            const double* __restrict__ blk, const double* __restrict__ r,
-                                            double* __restrict__ y) {
-  constexpr int NQ = K * (K + 1) / 2;
-  double m[NQ], rv[K];
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) m[q] = __ldcs(blk + q * n + s);
-#pragma unroll
-  for (int j = 0; j < K; ++j) rv[j] = __ldg(r + __ldg(mem + j * n + s));
-#pragma unroll
-  for (int i = 0; i < K; ++i) {
-    double v = 0.0;
-#pragma unroll
-    for (int j = 0; j < K; ++j) v = fma(m[i <= j ? upper(i, j, K) : upper(j, i, K)], rv[j], v);
-    y[i * n + s] = v;
-  }
-}
-
 __global__ void __launch_bounds__(256) k_schwarz_patch(SchwarzGroups g, int64_t npatch,
                                                        const int32_t* __restrict__ mem,
                                                        const double* __restrict__ blk, const double* __restrict__ r,
                                                        double* __restrict__ y) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= npatch) return;
-  const int k = group_of(g, t);
-  const int64_t s = t - g.first[k], n = g.count[k];
-  const int32_t* mm = mem + g.mbase[k];
-  const double* bb = blk + g.bbase[k];
-  double* yy = y + g.mbase[k];
-  switch (k) {  // uniform across a warp except at the group boundaries
-    case 1: patch_solve<1>(s, n, mm, bb, r, yy); break;
-    case 2: patch_solve<2>(s, n, mm, bb, r, yy); break;
-    case 3: patch_solve<3>(s, n, mm, bb, r, yy); break;
-    case 4: patch_solve<4>(s, n, mm, bb, r, yy); break;
-    case 5: patch_solve<5>(s, n, mm, bb, r, yy); break;
-    case 6: patch_solve<6>(s, n, mm, bb, r, yy); break;
-    case 7: patch_solve<7>(s, n, mm, bb, r, yy); break;
-    case 8: patch_solve<8>(s, n, mm, bb, r, yy); break;
-    default: {  // 9..kSchwarzDense members: rare; the block read entry by entry
-      double rv[kSchwarzDense];
-      for (int j = 0; j < k; ++j) rv[j] = __ldg(r + __ldg(mm + j * n + s));
-      for (int i = 0; i < k; ++i) {
-        double v = 0.0;
-        for (int j = 0; j < k; ++j) v = fma(__ldg(bb + (int64_t)(i <= j ? upper(i, j, k) : upper(j, i, k)) * n + s),
-                                            rv[j], v);
-        yy[i * n + s] = v;
-      }
-    }
-  }
+  patch_apply<true>(g, t, group_of(g, t), mem, blk, [r](int m) { return __ldg(r + m); }, y);
 }
 
 // z = sum of the three patch values of each multiplier (fixed order), r.z;
