@@ -65,12 +65,12 @@ __device__ __forceinline__ void misfit_load(const double* __restrict__ u, const 
 }
 
 // J partial sums: 1/2 e' M e = 1/2 |T|/20 (e.e + (sum e)^2)
-__global__ void __launch_bounds__(RT) k_misfit_partial(int64_t nE, const double* __restrict__ geo,
+__global__ void __launch_bounds__(RT) k_misfit_partial(int64_t nE, const double2* __restrict__ vol,
                                                        const double* __restrict__ u, const double* __restrict__ u_obs,
                                                        double* __restrict__ part) {
   double acc = 0.0;
   for (int64_t t = blockIdx.x * (int64_t)RT + threadIdx.x; t < nE; t += (int64_t)RB * RT) {
-    const double adet = __ldg(geo + PH_GEO_STRIDE * t + 15);
+    const double adet = __ldg(&vol[t].x);
     double e[4], r[4];
     misfit_load(u, u_obs, t, adet, e, r);
     acc = fma(0.5, (e[0] * r[0] + e[1] * r[1]) + (e[2] * r[2] + e[3] * r[3]), acc);
@@ -105,7 +105,7 @@ __device__ __forceinline__ void load_factor(const double* __restrict__ factor, i
 __device__ __forceinline__ int opp(int k) { return k == 0 ? 3 : (k == 3 ? 0 : k); }
 
 // rhs_q[l(F_k)] += -(C A^-1 r)_k
-__global__ void __launch_bounds__(128) k_adjoint_rhs(int64_t nE, const double* __restrict__ geo,
+__global__ void __launch_bounds__(128) k_adjoint_rhs(int64_t nE, const double2* __restrict__ vol,
                                                      const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                      const double* __restrict__ face_area,
                                                      const double* __restrict__ factor, double six_over_c,
@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(128) k_adjoint_rhs(int64_t nE, const double* _
                                                      double* __restrict__ rhs_q) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
-  const double* gp = geo + PH_GEO_STRIDE * t;
-  const double adet = __ldg(gp + 15), rdet = __ldg(gp + 16);
+  const double2 vt = __ldg(vol + t);
+  const double adet = vt.x, rdet = vt.y;
   double e[4], r[4];
   misfit_load(u, u_obs, t, adet, e, r);
   double Q[10];
@@ -143,6 +143,8 @@ __global__ void __launch_bounds__(128) k_adjoint_rhs(int64_t nE, const double* _
 
 // dJ/dtheta_T = -a_T/(6|det|) (D0 p)' adj(G_e) (D0 U)
 __global__ void __launch_bounds__(128) k_adjoint_grad(int64_t nE, const double* __restrict__ geo,
+                                                      const int32_t* __restrict__ gexp,
+                                                      const double2* __restrict__ vol,
                                                       const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                       const double* __restrict__ face_area,
                                                       const double* __restrict__ a,
@@ -151,7 +153,7 @@ __global__ void __launch_bounds__(128) k_adjoint_grad(int64_t nE, const double* 
                                                       const double* __restrict__ q, double* __restrict__ grad) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
-  const Geo G = load_geo(geo, t);
+  const Geo G = to_f64(load_record(geo, gexp, t), __ldg(vol + t));
   double e[4], r[4];
   misfit_load(u, u_obs, t, G.adet, e, r);
   double Q[10];
@@ -209,7 +211,7 @@ extern "C" ph_status ph_misfit(const ph_mesh* m, const double* u, const double* 
   double* part = nullptr;
   cudaError_t e = alloc(&part, RB, s);
   if (e != cudaSuccess) return cuda_status(e, "ph_misfit alloc");
-  k_misfit_partial<<<RB, RT, 0, s>>>(m->nE, m->geo, u, u_obs, part);
+  k_misfit_partial<<<RB, RT, 0, s>>>(m->nE, m->vol, u, u_obs, part);
   k_misfit_final<<<1, RT, 0, s>>>(part, J);
   e = launched(2);
   free_async(part, s);
@@ -228,7 +230,7 @@ extern "C" ph_status ph_adjoint_rhs(const ph_mesh* m, const double* factor, doub
     if (e != cudaSuccess) return cuda_status(e, "k_zero");
   }
   if (m->nE == 0) return PH_OK;
-  k_adjoint_rhs<<<grid_for(m->nE, 128), 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->face_area, factor, 6.0 / c,
+  k_adjoint_rhs<<<grid_for(m->nE, 128), 128, 0, s>>>(m->nE, m->vol, m->tface, m->tmult, m->face_area, factor, 6.0 / c,
                                                      u, u_obs, rhs_q);
   return cuda_status(launched(), "k_adjoint_rhs");
 }
@@ -244,7 +246,7 @@ extern "C" ph_status ph_adjoint_grad(const ph_mesh* m, const double* a, const do
   if (m->nE > 0 && (!a || !factor || !u || !u_obs || !grad || (m->L > 0 && !q))) return PH_ERR_ARG;
   if (m->nE == 0) return PH_OK;
   cudaStream_t s = (cudaStream_t)stream;
-  k_adjoint_grad<<<grid_for(m->nE, 128), 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->face_area, a, factor,
+  k_adjoint_grad<<<grid_for(m->nE, 128), 128, 0, s>>>(m->nE, m->geo, m->gexp, m->vol, m->tface, m->tmult, m->face_area, a, factor,
                                                       6.0 / c, u, u_obs, q, grad);
   return cuda_status(launched(), "k_adjoint_grad");
 }

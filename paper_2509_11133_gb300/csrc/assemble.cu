@@ -23,8 +23,9 @@
 // (the load B_j = sum_k h'_k/3 [j != o(k)] is the paper's face-centroid rule),
 // and recovery U(T) = A^-1 (B + C' Lambda_T) is
 //     U[o(k)] = z'sum/(c|T|) - (Qf z')_k / 3,   z'_k = h'_k + d_k Lambda_k.
-// G_e and G_e T0^-1 come precomputed per element from the mesh (they depend
-// on the geometry only).  ph_assemble can also store Qf/9 per element (the
+// G_e comes precomputed per element from the mesh (it depends on the geometry
+// only), and the 3x3 algebra runs in fixed point on the integer pipe
+// (fixed.cuh), or in fp64 for the elements that leaves out.  ph_assemble can also store Qf/9 per element (the
 // "element factor", 10 numbers) so that ph_recover_factored skips the
 // condensation kernel.
 #include <math.h>
@@ -37,8 +38,13 @@ using namespace ph_elem;
 
 namespace {
 
-template <bool UD, bool GN, bool FAC, int MODE>
-__global__ void __launch_bounds__(128, MODE ? 7 : 1) k_assemble(int64_t nE, const double* __restrict__ geo,
+// Fixed-point kernel: 58 FP64 operations per element where fp64 took 114 (17.9M
+// tets: 3.70 -> 2.31 ms; the FP64 pipe alone needs 1.9).  Six blocks of 128
+// threads per SM (80 registers): 4 (122 registers), 5 and 7 take 2.70, 2.40
+// and 2.31 ms.
+template <bool UD, bool GN, bool FAC, bool DW>
+__global__ void __launch_bounds__(128, DW ? 7 : 6) k_assemble(int64_t nE, const double* __restrict__ geo,
+                                                  const int32_t* __restrict__ gexp, const double2* __restrict__ vol,
                                                   const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                   const int4* __restrict__ tpos, const ushort4* __restrict__ trel,
                                                   const double* __restrict__ face_area, const double* __restrict__ a,
@@ -49,13 +55,14 @@ __global__ void __launch_bounds__(128, MODE ? 7 : 1) k_assemble(int64_t nE, cons
                                                   const double* __restrict__ coord, const int4* __restrict__ tet) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
-  assemble_element<UD, GN, FAC, MODE>(t, geo, tface, tmult, tpos, trel, face_area, a, c20, six_over_c, f_face, uD,
+  assemble_element<UD, GN, FAC, DW>(t, geo, gexp, vol, tface, tmult, tpos, trel, face_area, a, c20, six_over_c, f_face, uD,
                                       gN, values, rhs, factor, status, coord, tet);
 }
 
 
 template <bool GN>
 __global__ void __launch_bounds__(128) k_recover(int64_t nE, const double* __restrict__ geo,
+                                                 const int32_t* __restrict__ gexp, const double2* __restrict__ vol,
                                                  const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                  const double* __restrict__ face_area, const double* __restrict__ a,
                                                  double c20, double six_over_c, const double* __restrict__ f_face,
@@ -68,27 +75,28 @@ __global__ void __launch_bounds__(128) k_recover(int64_t nE, const double* __res
     ph_flag(status, PH_ERR_ARG);
     return;
   }
-  const Geo G = load_geo(geo, t);
+  const double2 vt = __ldg(vol + t);
+  const Record R = load_record(geo, gexp, t);
   double z[4];
-  recovery_load<GN>(G.adet * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
+  recovery_load<GN>(vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
   double Q[10];
-  face_kernel(G, at, c20, -6.0 / 3.0, Q);  // -Qf/3
-  const double icT = G.rdet * six_over_c;
+  element_kernel(R, vt, at, c20, Q);  // Qf/9
+  const double icT = vt.y * six_over_c;
   const double zs = icT * ((z[0] + z[1]) + (z[2] + z[3]));
   double U[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    double e = zs;
+    double e = 0.0;
 #pragma unroll
     for (int m = 0; m < 4; ++m) e = fma(Q[ut(k, m)], z[m], e);
-    U[k] = e;
+    U[k] = fma(-3.0, e, zs);
   }
   store_u(u, t, U);
 }
 
 // Recovery from the element factor Qf/9 stored by ph_assemble.
 template <bool GN>
-__global__ void __launch_bounds__(128) k_recover_factored(int64_t nE, const double* __restrict__ geo,
+__global__ void __launch_bounds__(128) k_recover_factored(int64_t nE, const double2* __restrict__ vol,
                                                           const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                           const double* __restrict__ face_area,
                                                           const double* __restrict__ factor, double six_over_c,
@@ -97,7 +105,7 @@ __global__ void __launch_bounds__(128) k_recover_factored(int64_t nE, const doub
                                                           const double* __restrict__ lambda, double* __restrict__ u) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
-  recover_element_factored<GN>(t, geo, tface, tmult, face_area, factor, six_over_c, f_face, gN, lambda, u);
+  recover_element_factored<GN>(t, vol, tface, tmult, face_area, factor, six_over_c, f_face, gN, lambda, u);
 }
 
 bool finite_pos(double x) { return x > 0.0 && x < INFINITY; }
@@ -116,13 +124,13 @@ static bool needs_fp64_record(const ph_mesh* m, const char* who) {
   return true;
 }
 
-template <int MODE>
+template <bool DW>
 static void launch_assemble(const ph_mesh* m, unsigned grid, bool ud, bool gn, double c20, double six_over_c,
                             const double* a, const double* f_face, const double* uD_face, const double* gN_face,
                             double* values, double* rhs, double* factor, cudaStream_t s) {
 #define PH_ASM(UDV, GNV, FACV)                                                                                  \
-  k_assemble<UDV, GNV, FACV, MODE><<<grid, 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->tpos, m->trel,   \
-                                                        m->face_area, a, c20, six_over_c, f_face, uD_face,     \
+  k_assemble<UDV, GNV, FACV, DW><<<grid, 128, 0, s>>>(m->nE, m->geo, m->gexp, m->vol, m->tface, m->tmult,       \
+                                                      m->tpos, m->trel, m->face_area, a, c20, six_over_c, f_face, uD_face,     \
                                                         gN_face, values, rhs, factor, m->status, m->coord, m->tet)
   if (factor) {
     if (ud && gn) PH_ASM(true, true, true);
@@ -162,12 +170,10 @@ static ph_status assemble(const ph_mesh* m, const double* a, double c, const dou
   const unsigned grid = grid_for(m->nE, 128);
   const bool ud = uD_face != nullptr && m->nFd > 0, gn = gN_face != nullptr && m->nFn > 0;
   KernelTimer kt(DW ? "k_assemble_dw" : "k_assemble", s);
-  if (!DW)
-    launch_assemble<0>(m, grid, ud, gn, c20, six_over_c, a, f_face, uD_face, gN_face, values, rhs, factor, s);
-  else if (!m->geo_dw)
-    launch_assemble<1>(m, grid, ud, gn, c20, six_over_c, a, f_face, uD_face, gN_face, values, rhs, factor, s);
+  if (m->geo_dw)
+    launch_assemble<true>(m, grid, ud, gn, c20, six_over_c, a, f_face, uD_face, gN_face, values, rhs, factor, s);
   else
-    launch_assemble<2>(m, grid, ud, gn, c20, six_over_c, a, f_face, uD_face, gN_face, values, rhs, factor, s);
+    launch_assemble<false>(m, grid, ud, gn, c20, six_over_c, a, f_face, uD_face, gN_face, values, rhs, factor, s);
   const cudaError_t e = launched();
   kt.stop();
   return cuda_status(e, "k_assemble");
@@ -180,7 +186,7 @@ extern "C" ph_status ph_assemble(const ph_mesh* m, const double* a, double c, co
 }
 
 template <bool GN>
-__global__ void __launch_bounds__(128) k_recover_factored_dw(int64_t nE, const double* __restrict__ geo,
+__global__ void __launch_bounds__(128) k_recover_factored_dw(int64_t nE, const double2* __restrict__ vol,
                                                              const int4* __restrict__ tface,
                                                              const int4* __restrict__ tmult,
                                                              const double* __restrict__ face_area,
@@ -191,7 +197,7 @@ __global__ void __launch_bounds__(128) k_recover_factored_dw(int64_t nE, const d
                                                              double* __restrict__ u) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
-  recover_element_factored_dw<GN>(t, geo, tface, tmult, face_area, factor, six_over_c, f_face, gN, lambda, u);
+  recover_element_factored_dw<GN>(t, vol, tface, tmult, face_area, factor, six_over_c, f_face, gN, lambda, u);
 }
 
 extern "C" ph_status ph_assemble_dw(const ph_mesh* m, const double* a, double c, const double* f_face,
@@ -211,10 +217,10 @@ extern "C" ph_status ph_recover(const ph_mesh* m, const double* a, double c, con
   const unsigned grid = grid_for(m->nE, 128);
   KernelTimer kt("k_recover", s);
   if (gN_face != nullptr && m->nFn > 0)
-    k_recover<true><<<grid, 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->face_area, a, c20, six_over_c, f_face,
+    k_recover<true><<<grid, 128, 0, s>>>(m->nE, m->geo, m->gexp, m->vol, m->tface, m->tmult, m->face_area, a, c20, six_over_c, f_face,
                                          gN_face, lambda, u, m->status);
   else
-    k_recover<false><<<grid, 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->face_area, a, c20, six_over_c,
+    k_recover<false><<<grid, 128, 0, s>>>(m->nE, m->geo, m->gexp, m->vol, m->tface, m->tmult, m->face_area, a, c20, six_over_c,
                                           f_face, gN_face, lambda, u, m->status);
   const cudaError_t e = launched();
   kt.stop();
@@ -231,10 +237,10 @@ extern "C" ph_status ph_recover_factored(const ph_mesh* m, const double* factor,
   const unsigned grid = grid_for(m->nE, 128);
   KernelTimer kt("k_recover_factored", s);
   if (gN_face != nullptr && m->nFn > 0)
-    k_recover_factored<true><<<grid, 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->face_area, factor,
+    k_recover_factored<true><<<grid, 128, 0, s>>>(m->nE, m->vol, m->tface, m->tmult, m->face_area, factor,
                                                   six_over_c, f_face, gN_face, lambda, u);
   else
-    k_recover_factored<false><<<grid, 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->face_area, factor,
+    k_recover_factored<false><<<grid, 128, 0, s>>>(m->nE, m->vol, m->tface, m->tmult, m->face_area, factor,
                                                    six_over_c, f_face, gN_face, lambda, u);
   const cudaError_t e = launched();
   kt.stop();
@@ -251,10 +257,10 @@ extern "C" ph_status ph_recover_factored_dw(const ph_mesh* m, const double* fact
   const unsigned grid = grid_for(m->nE, 128);
   KernelTimer kt("k_recover_factored_dw", s);
   if (gN_face != nullptr && m->nFn > 0)
-    k_recover_factored_dw<true><<<grid, 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->face_area, factor,
+    k_recover_factored_dw<true><<<grid, 128, 0, s>>>(m->nE, m->vol, m->tface, m->tmult, m->face_area, factor,
                                                      six_over_c, f_face, gN_face, lambda, u);
   else
-    k_recover_factored_dw<false><<<grid, 128, 0, s>>>(m->nE, m->geo, m->tface, m->tmult, m->face_area, factor,
+    k_recover_factored_dw<false><<<grid, 128, 0, s>>>(m->nE, m->vol, m->tface, m->tmult, m->face_area, factor,
                                                       six_over_c, f_face, gN_face, lambda, u);
   const cudaError_t e = launched();
   kt.stop();

@@ -25,6 +25,8 @@ namespace {
 
 struct ProbDesc {
   const double* geo;
+  const int32_t* gexp;
+  const double2* vol;
   const int4* tface;
   const int4* tmult;
   const int4* tpos;
@@ -56,7 +58,7 @@ struct Tile {
 template <bool UD, bool GN, bool FAC>
 __device__ __forceinline__ void run_tile(const ProbDesc& d, int64_t start, int count) {
   for (int i = threadIdx.x; i < count; i += blockDim.x)
-    assemble_element<UD, GN, FAC>(start + i, d.geo, d.tface, d.tmult, d.tpos, d.trel, d.area, d.a, d.c20,
+    assemble_element<UD, GN, FAC>(start + i, d.geo, d.gexp, d.vol, d.tface, d.tmult, d.tpos, d.trel, d.area, d.a, d.c20,
                                   d.six_over_c, d.f, d.uD, d.gN, d.values, d.rhs, d.factor, d.status);
 }
 
@@ -87,10 +89,10 @@ __global__ void k_batch_recover(const ProbDesc* __restrict__ probs, const Tile* 
     if (!d.u) continue;
     for (int i = threadIdx.x; i < tl.count; i += blockDim.x) {
       if (d.flags & 2)
-        recover_element_factored<true>(tl.start + i, d.geo, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f,
+        recover_element_factored<true>(tl.start + i, d.vol, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f,
                                        d.gN, d.lambda, d.u);
       else
-        recover_element_factored<false>(tl.start + i, d.geo, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f,
+        recover_element_factored<false>(tl.start + i, d.vol, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f,
                                         d.gN, d.lambda, d.u);
     }
   }
@@ -243,6 +245,8 @@ extern "C" ph_status ph_batch_bind(ph_batch* b, const double* const* a, const do
     d.lambda = keep_lambda;
     d.u = keep_u;
     d.geo = m->geo;
+    d.gexp = m->gexp;
+    d.vol = m->vol;
     d.tface = m->tface;
     d.tmult = m->tmult;
     d.tpos = m->tpos;

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "dw.cuh"
+#include "fixed.cuh"
 #include "ph_internal.cuh"
 
 namespace ph_elem {
@@ -20,52 +21,60 @@ __host__ __device__ constexpr int ut(int k, int m) {
 
 struct Geo {
   double g00, g01, g02, g11, g12, g22;  // G_e
-  double t00, t01, t02, t10, t11, t12, t20, t21, t22;  // G_e T0^-1
   double adet, rdet;
 };
 
-// Element geometry of tet [P0 P1 P2 P3] in fp64: E = rows P_i - P_0
-// (i = 1..3), G_e = E E', GT = G_e T0^-1 = G_e - (G_e 1) 1'/4 (T0 = I + 1 1';
-// one fma per entry, the quarter being exact), |det E| and 1/|det E| (the
-// Newton reciprocal).  The mesh build stores it as the element's fp64
-// record; the double-word kernels recompute it for elements they hand to the
-// fp64 path.
-__device__ __forceinline__ Geo compute_geo(const double* __restrict__ coord, int4 v) {
+// The edge vectors E = rows P_i - P_0 (i = 1..3) of tet [P0 P1 P2 P3].
+__device__ __forceinline__ void edge_vectors(const double* __restrict__ coord, int4 v, double e[3][3]) {
   const double* p0 = coord + 3 * (int64_t)v.x;
   const double* p1 = coord + 3 * (int64_t)v.y;
   const double* p2 = coord + 3 * (int64_t)v.z;
   const double* p3 = coord + 3 * (int64_t)v.w;
-  const double e1x = p1[0] - p0[0], e1y = p1[1] - p0[1], e1z = p1[2] - p0[2];
-  const double e2x = p2[0] - p0[0], e2y = p2[1] - p0[1], e2z = p2[2] - p0[2];
-  const double e3x = p3[0] - p0[0], e3y = p3[1] - p0[1], e3z = p3[2] - p0[2];
-  const double det = e1x * (e2y * e3z - e2z * e3y) + e1y * (e2z * e3x - e2x * e3z) + e1z * (e2x * e3y - e2y * e3x);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    e[0][d] = p1[d] - p0[d];
+    e[1][d] = p2[d] - p0[d];
+    e[2][d] = p3[d] - p0[d];
+  }
+}
+
+// Element geometry in fp64: G_e = E E', |det E| and 1/|det E| (the Newton
+// reciprocal), for the elements that fx::geometry leaves to fp64 and those the
+// double-word kernel hands to the fp64 path.
+__device__ __forceinline__ Geo compute_geo(const double e[3][3]) {
+  const double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) +
+                     e[0][1] * (e[1][2] * e[2][0] - e[1][0] * e[2][2]) +
+                     e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
   Geo G;
   G.adet = ph::neg_if(det, __double2hiint(det) < 0);  // |det| on the sign bit
-  G.g00 = e1x * e1x + e1y * e1y + e1z * e1z;
-  G.g01 = e1x * e2x + e1y * e2y + e1z * e2z;
-  G.g02 = e1x * e3x + e1y * e3y + e1z * e3z;
-  G.g11 = e2x * e2x + e2y * e2y + e2z * e2z;
-  G.g12 = e2x * e3x + e2y * e3y + e2z * e3z;
-  G.g22 = e3x * e3x + e3y * e3y + e3z * e3z;
-  const double r0 = (G.g00 + G.g01) + G.g02, r1 = (G.g01 + G.g11) + G.g12, r2 = (G.g02 + G.g12) + G.g22;
-  G.t00 = fma(-0.25, r0, G.g00);
-  G.t01 = fma(-0.25, r0, G.g01);
-  G.t02 = fma(-0.25, r0, G.g02);
-  G.t10 = fma(-0.25, r1, G.g01);
-  G.t11 = fma(-0.25, r1, G.g11);
-  G.t12 = fma(-0.25, r1, G.g12);
-  G.t20 = fma(-0.25, r2, G.g02);
-  G.t21 = fma(-0.25, r2, G.g12);
-  G.t22 = fma(-0.25, r2, G.g22);
+  G.g00 = e[0][0] * e[0][0] + e[0][1] * e[0][1] + e[0][2] * e[0][2];
+  G.g01 = e[0][0] * e[1][0] + e[0][1] * e[1][1] + e[0][2] * e[1][2];
+  G.g02 = e[0][0] * e[2][0] + e[0][1] * e[2][1] + e[0][2] * e[2][2];
+  G.g11 = e[1][0] * e[1][0] + e[1][1] * e[1][1] + e[1][2] * e[1][2];
+  G.g12 = e[1][0] * e[2][0] + e[1][1] * e[2][1] + e[1][2] * e[2][2];
+  G.g22 = e[2][0] * e[2][0] + e[2][1] * e[2][1] + e[2][2] * e[2][2];
   G.rdet = ph::rcp_newton(G.adet);
   return G;
 }
 
-__device__ __forceinline__ Geo load_geo(const double* __restrict__ geo, int64_t t) {
-  const double2* p = reinterpret_cast<const double2*>(geo + PH_GEO_STRIDE * t);
-  const double2 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2), d = __ldg(p + 3), e = __ldg(p + 4);
-  const double2 f = __ldg(p + 5), g = __ldg(p + 6), h = __ldg(p + 7), i = __ldg(p + 8);
-  return Geo{a.x, a.y, b.x, b.y, c.x, c.y, d.x, d.y, e.x, e.y, f.x, f.y, g.x, g.y, h.x, h.y, i.x};
+// The geometry record of element t as stored: g and its scale.
+struct Record {
+  int64_t g[6];
+  int kg;  // PH_GEXP_F64: g holds doubles
+};
+__device__ __forceinline__ Record load_record(const double* __restrict__ geo, const int32_t* __restrict__ gexp,
+                                              int64_t t) {
+  const longlong2* p = reinterpret_cast<const longlong2*>(geo + PH_GEO_STRIDE * t);
+  const longlong2 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+  return Record{{a.x, a.y, b.x, b.y, c.x, c.y}, __ldg(gexp + t)};
+}
+// The same in fp64.
+__device__ __forceinline__ Geo to_f64(const Record& r, double2 vol) {
+  double g[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+    g[i] = r.kg == PH_GEXP_F64 ? __longlong_as_double(r.g[i]) : fx::to_double(r.g[i], r.kg);
+  return Geo{g[0], g[1], g[2], g[3], g[4], g[5], vol.x, vol.y};
 }
 
 // Qf (face-indexed, packed upper triangle) times sc = sc6/6.
@@ -82,13 +91,18 @@ __device__ __forceinline__ void face_kernel(const Geo& G, double a, double c20, 
   const double detM = fma(m00, A00, fma(m01, A01, m02 * A02));
   const double s = (sc6 * G.rdet) * ph::rcp_newton(detM);  // sc * 6/|det E| / det M
   A00 *= s; A01 *= s; A02 *= s; A11 *= s; A12 *= s; A22 *= s;
+  // G_e T0^-1 = G_e - (G_e 1) 1'/4 (T0 = I + 1 1'; one fma per entry, the quarter being exact)
+  const double r0 = (G.g00 + G.g01) + G.g02, r1 = (G.g01 + G.g11) + G.g12, r2 = (G.g02 + G.g12) + G.g22;
+  const double t00 = fma(-0.25, r0, G.g00), t01 = fma(-0.25, r0, G.g01), t02 = fma(-0.25, r0, G.g02);
+  const double t10 = fma(-0.25, r1, G.g01), t11 = fma(-0.25, r1, G.g11), t12 = fma(-0.25, r1, G.g12);
+  const double t20 = fma(-0.25, r2, G.g02), t21 = fma(-0.25, r2, G.g12), t22 = fma(-0.25, r2, G.g22);
   // Y = adj(M) G_e T0^-1 (symmetric): upper triangle
-  const double y00 = fma(A00, G.t00, fma(A01, G.t10, A02 * G.t20));
-  const double y01 = fma(A00, G.t01, fma(A01, G.t11, A02 * G.t21));
-  const double y02 = fma(A00, G.t02, fma(A01, G.t12, A02 * G.t22));
-  const double y11 = fma(A01, G.t01, fma(A11, G.t11, A12 * G.t21));
-  const double y12 = fma(A01, G.t02, fma(A11, G.t12, A12 * G.t22));
-  const double y22 = fma(A02, G.t02, fma(A12, G.t12, A22 * G.t22));
+  const double y00 = fma(A00, t00, fma(A01, t10, A02 * t20));
+  const double y01 = fma(A00, t01, fma(A01, t11, A02 * t21));
+  const double y02 = fma(A00, t02, fma(A01, t12, A02 * t22));
+  const double y11 = fma(A01, t01, fma(A11, t11, A12 * t21));
+  const double y12 = fma(A01, t02, fma(A11, t12, A12 * t22));
+  const double y22 = fma(A02, t02, fma(A12, t12, A22 * t22));
   // Qv = D0' Y D0; faces 0,1,2,3 sit opposite vertices 3,1,2,0
   const double c0 = y00 + y01 + y02, c1 = y01 + y11 + y12, c2 = y02 + y12 + y22;
   Q[ut(0, 0)] = y22;
@@ -103,6 +117,14 @@ __device__ __forceinline__ void face_kernel(const Geo& G, double a, double c20, 
   Q[ut(3, 3)] = c0 + c1 + c2;
 }
 
+// The condensation kernel Qf/9 of an element from its record: fixed point
+// (fixed.cuh), or fp64 for the elements it leaves out.
+__device__ __forceinline__ void element_kernel(const Record& r, double2 vol, double a, double c20, double Q[10]) {
+  const auto rcp = [](double x) { return ph::rcp_newton(x); };
+  if (r.kg == PH_GEXP_F64 || !fx::face_kernel(r.g, r.kg, a, c20, vol.y, rcp, Q))
+    face_kernel(to_f64(r, vol), a, c20, 6.0 / 9.0, Q);
+}
+
 // The geometry of one element in double-word form: G' = 2^-kg G_e and
 // G'T = 2^-kg G_e T0^-1, 2^kg the binade of the largest diagonal entry of
 // G_e (so every value is below ~8 in magnitude), |det E| and 1/|det E| in
@@ -115,39 +137,11 @@ struct GeoDW {
   int kg, flat;
 };
 
-// The double-word geometry from the fp64 record (integer conversions).
-__device__ __forceinline__ GeoDW geo_dw_from(const Geo& G) {
-  using namespace dw;
-  GeoDW D;
-  const int e0 = exponent(G.g00), e1 = exponent(G.g11), e2 = exponent(G.g22);
-  D.kg = max(e0, max(e1, e2));
-  D.flat = -2 * exponent(G.rdet) - (e0 + e1 + e2);
-  const int s = -D.kg;
-  D.g[0] = from_double(G.g00, s);
-  D.g[1] = from_double(G.g01, s);
-  D.g[2] = from_double(G.g02, s);
-  D.g[3] = from_double(G.g11, s);
-  D.g[4] = from_double(G.g12, s);
-  D.g[5] = from_double(G.g22, s);
-  D.t[0] = from_double(G.t00, s);
-  D.t[1] = from_double(G.t01, s);
-  D.t[2] = from_double(G.t02, s);
-  D.t[3] = from_double(G.t10, s);
-  D.t[4] = from_double(G.t11, s);
-  D.t[5] = from_double(G.t12, s);
-  D.t[6] = from_double(G.t20, s);
-  D.t[7] = from_double(G.t21, s);
-  D.t[8] = from_double(G.t22, s);
-  D.adet = G.adet;
-  D.rdet = G.rdet;
-  return D;
-}
-
-// The double-word record of a mesh built by ph_mesh_create_dw (same 144 bytes
-// per element as the fp64 record: 30 floats of pairs, then |det E| and
+// The double-word record of a mesh built by ph_mesh_create_dw (144 bytes per
+// element: 30 floats of pairs, then |det E| and
 // 1/|det E| as doubles 15 and 16, then kg and the flatness as two ints).
 __device__ __forceinline__ GeoDW load_geo_dw(const double* __restrict__ geo, int64_t t) {
-  const float4* p = reinterpret_cast<const float4*>(geo + PH_GEO_STRIDE * t);
+  const float4* p = reinterpret_cast<const float4*>(geo + PH_GEO_DW_STRIDE * t);
   float v[36];
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
@@ -249,12 +243,12 @@ using ph::neg_if;
 
 // Local matrices, condensation and scatter of element t (Section 4.2-4.3,
 // Eq. schur): the body of the assembly kernels (one thread per element).
-// MODE: 0 fp64 (the fp64 record, face_kernel); 1 the double-word face
-// kernel on the fp64 record (converted); 2 the double-word record of a mesh
-// from ph_mesh_create_dw (elements the double-word kernel hands back get
-// their fp64 geometry recomputed from coord and tet).
-template <bool UD, bool GN, bool FAC, int MODE = 0>
+// DW: the double-word record of a mesh from ph_mesh_create_dw (elements the
+// double-word kernel hands back get their fp64 geometry recomputed from coord
+// and tet); else the fixed-point record.
+template <bool UD, bool GN, bool FAC, bool DW = false>
 __device__ __forceinline__ void assemble_element(int64_t t, const double* __restrict__ geo,
+                                                 const int32_t* __restrict__ gexp, const double2* __restrict__ vol,
                                                  const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                  const int4* __restrict__ tpos, const ushort4* __restrict__ trel,
                                                  const double* __restrict__ face_area, const double* __restrict__ a,
@@ -269,16 +263,11 @@ __device__ __forceinline__ void assemble_element(int64_t t, const double* __rest
     ph_flag(status, PH_ERR_ARG);
     return;
   }
-  Geo G;
+  const double2 vt = __ldg(vol + t);  // |det E|, 1/|det E|
+  Record R;
   GeoDW D;
-  if (MODE == 2) {
-    D = load_geo_dw(geo, t);
-    G.adet = D.adet;
-    G.rdet = D.rdet;
-  } else {
-    G = load_geo(geo, t);
-    if (MODE == 1) D = geo_dw_from(G);
-  }
+  if (DW) D = load_geo_dw(geo, t);
+  else R = load_record(geo, gexp, t);
   const int4 tf = __ldg(tface + t);
   const int4 tm = __ldg(tmult + t);
   int F[4];
@@ -290,18 +279,19 @@ __device__ __forceinline__ void assemble_element(int64_t t, const double* __rest
     neg[k] = comp(tf, k) < 0;
     ar[k] = __ldg(face_area + F[k]);
   }
-  const double q4 = G.adet * (1.0 / 24.0);  // |T| / 4
+  const double q4 = vt.x * (1.0 / 24.0);  // |T| / 4
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     h[k] = q4 * __ldg(f_face + F[k]);
     if (GN && comp(tm, k) == PH_NO_MULT) h[k] = fma(ar[k], __ldg(gN + F[k]), h[k]);
   }
   double Q[10];
-  if (MODE == 0) {
-    face_kernel(G, at, c20, 6.0 / 9.0, Q);
+  if (!DW) {
+    element_kernel(R, vt, at, c20, Q);
   } else if (!face_kernel_dw(D, at, c20, 6.0 / 9.0, Q)) {
-    if (MODE == 2) G = compute_geo(coord, __ldg(tet + t));
-    face_kernel(G, at, c20, 6.0 / 9.0, Q);
+    double e[3][3];
+    edge_vectors(coord, __ldg(tet + t), e);
+    face_kernel(compute_geo(e), at, c20, 6.0 / 9.0, Q);
   }
   if (FAC) {
     double2* fo = reinterpret_cast<double2*>(factor + 10 * t);
@@ -311,7 +301,7 @@ __device__ __forceinline__ void assemble_element(int64_t t, const double* __rest
     fo[3] = make_double2(Q[6], Q[7]);
     fo[4] = make_double2(Q[8], Q[9]);
   }
-  const double icT = G.rdet * six_over_c;  // 1/(c|T|)
+  const double icT = vt.y * six_over_c;  // 1/(c|T|)
   const double hs = (h[0] + h[1]) + (h[2] + h[3]);
   const double base = icT * hs;
   // condensed block S[k][m] = d_k d_m (1/(c|T|) + Qf/9), each entry once, as
@@ -395,7 +385,7 @@ __device__ __forceinline__ void recovery_load(double q4, int4 tf, int4 tm, const
 // (Algorithm 1, second loop): U[o(k)] = z'sum/(c|T|) - 3 (Qf/9 z')_k.  The
 // body of the plain and the batched recovery kernels.
 template <bool GN>
-__device__ __forceinline__ void recover_element_factored(int64_t t, const double* __restrict__ geo,
+__device__ __forceinline__ void recover_element_factored(int64_t t, const double2* __restrict__ vol,
                                                          const int4* __restrict__ tface,
                                                          const int4* __restrict__ tmult,
                                                          const double* __restrict__ face_area,
@@ -403,14 +393,13 @@ __device__ __forceinline__ void recover_element_factored(int64_t t, const double
                                                          const double* __restrict__ f_face,
                                                          const double* __restrict__ gN,
                                                          const double* __restrict__ lambda, double* __restrict__ u) {
-  const double2 dr = __ldg(reinterpret_cast<const double2*>(geo + PH_GEO_STRIDE * t) + 7);  // (t22, |det|)
-  const double rdet = __ldg(geo + PH_GEO_STRIDE * t + 16);
+  const double2 vt = __ldg(vol + t);
   double z[4];
-  recovery_load<GN>(dr.y * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
+  recovery_load<GN>(vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
   const double2* fp = reinterpret_cast<const double2*>(factor + 10 * t);
   const double2 q0 = __ldg(fp), q1 = __ldg(fp + 1), q2 = __ldg(fp + 2), q3 = __ldg(fp + 3), q4 = __ldg(fp + 4);
   const double Q[10] = {q0.x, q0.y, q1.x, q1.y, q2.x, q2.y, q3.x, q3.y, q4.x, q4.y};
-  const double icT = rdet * six_over_c;
+  const double icT = vt.y * six_over_c;
   const double zs = icT * ((z[0] + z[1]) + (z[2] + z[3]));
   double U[4];
 #pragma unroll
@@ -433,7 +422,7 @@ __device__ __forceinline__ void recover_element_factored(int64_t t, const double
 // instead of 34.  Elements whose binades leave the pairs' range take the fp64
 // product.
 template <bool GN>
-__device__ __forceinline__ void recover_element_factored_dw(int64_t t, const double* __restrict__ geo,
+__device__ __forceinline__ void recover_element_factored_dw(int64_t t, const double2* __restrict__ vol,
                                                             const int4* __restrict__ tface,
                                                             const int4* __restrict__ tmult,
                                                             const double* __restrict__ face_area,
@@ -443,14 +432,13 @@ __device__ __forceinline__ void recover_element_factored_dw(int64_t t, const dou
                                                             const double* __restrict__ lambda,
                                                             double* __restrict__ u) {
   using namespace dw;
-  const double2 dr = __ldg(reinterpret_cast<const double2*>(geo + PH_GEO_STRIDE * t) + 7);  // (t22, |det|)
-  const double rdet = __ldg(geo + PH_GEO_STRIDE * t + 16);
+  const double2 vt = __ldg(vol + t);
   double z[4];
-  recovery_load<GN>(dr.y * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
+  recovery_load<GN>(vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
   const double2* fp = reinterpret_cast<const double2*>(factor + 10 * t);
   const double2 q0 = __ldg(fp), q1 = __ldg(fp + 1), q2 = __ldg(fp + 2), q3 = __ldg(fp + 3), q4 = __ldg(fp + 4);
   const double Q[10] = {q0.x, q0.y, q1.x, q1.y, q2.x, q2.y, q3.x, q3.y, q4.x, q4.y};
-  const double icT = rdet * six_over_c;
+  const double icT = vt.y * six_over_c;
   const double zs = icT * ((z[0] + z[1]) + (z[2] + z[3]));
   int kq = -1023, kz = -1023;
 #pragma unroll

@@ -72,22 +72,33 @@ __device__ __forceinline__ int64_t bucket_of(int3 s, int sub) {
   return ((int64_t)s.z << sub) | ((s.x ^ s.y) & ((1 << sub) - 1));
 }
 
-// Element geometry record of tet t (fp64; compute_geo): G_e, G_e T0^-1,
-// |det E|, 1/|det E|.
+// Element geometry of tet t: the record (G_e, fixed point or fp64), its scale,
+// |det E| and 1/|det E|.
 __device__ __forceinline__ void tet_geom(const double* __restrict__ coord, int4 v, int64_t t,
-                                         double* __restrict__ geo, unsigned* status) {
-  const ph_elem::Geo G = ph_elem::compute_geo(coord, v);
-  if (!ph::pos_finite(G.adet)) ph_flag(status, PH_ERR_DEGENERATE);
-  double2* gg = reinterpret_cast<double2*>(geo + PH_GEO_STRIDE * t);
-  gg[0] = make_double2(G.g00, G.g01);
-  gg[1] = make_double2(G.g02, G.g11);
-  gg[2] = make_double2(G.g12, G.g22);
-  gg[3] = make_double2(G.t00, G.t01);
-  gg[4] = make_double2(G.t02, G.t10);
-  gg[5] = make_double2(G.t11, G.t12);
-  gg[6] = make_double2(G.t20, G.t21);
-  gg[7] = make_double2(G.t22, G.adet);
-  gg[8] = make_double2(G.rdet, 0.0);
+                                         double* __restrict__ geo, int32_t* __restrict__ gexp,
+                                         double2* __restrict__ vol, unsigned* status) {
+  double e[3][3];
+  ph_elem::edge_vectors(coord, v, e);
+  ph_elem::Record r;
+  double adet, rdet;
+  if (fx::geometry(e, r.g, r.kg, adet)) {
+    rdet = ph::rcp_newton(adet);
+  } else {
+    const ph_elem::Geo G = ph_elem::compute_geo(e);
+    if (!ph::pos_finite(G.adet)) ph_flag(status, PH_ERR_DEGENERATE);
+    const double g[6] = {G.g00, G.g01, G.g02, G.g11, G.g12, G.g22};
+#pragma unroll
+    for (int i = 0; i < 6; ++i) r.g[i] = __double_as_longlong(g[i]);
+    r.kg = PH_GEXP_F64;
+    adet = G.adet;
+    rdet = G.rdet;
+  }
+  longlong2* o = reinterpret_cast<longlong2*>(geo + PH_GEO_STRIDE * t);
+  o[0] = make_longlong2(r.g[0], r.g[1]);
+  o[1] = make_longlong2(r.g[2], r.g[3]);
+  o[2] = make_longlong2(r.g[4], r.g[5]);
+  gexp[t] = r.kg;
+  vol[t] = make_double2(adet, rdet);
 }
 
 // The double-word geometry record of tet t (meshes of ph_mesh_create_dw):
@@ -96,19 +107,10 @@ __device__ __forceinline__ void tet_geom(const double* __restrict__ coord, int4 
 // of its largest entry, G' = E'E'^T, its scale 2^kg and G'T = G' - (G' 1) 1'/4
 // in double-word (dw.cuh), stored as the layout of load_geo_dw reads it.
 __device__ __forceinline__ void tet_geom_dw(const double* __restrict__ coord, int4 v, int64_t t,
-                                            double* __restrict__ geo, unsigned* status) {
+                                            double* __restrict__ geo, double2* __restrict__ vol, unsigned* status) {
   using namespace dw;
-  const double* p0 = coord + 3 * (int64_t)v.x;
-  const double* p1 = coord + 3 * (int64_t)v.y;
-  const double* p2 = coord + 3 * (int64_t)v.z;
-  const double* p3 = coord + 3 * (int64_t)v.w;
   double e[3][3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    e[0][d] = p1[d] - p0[d];
-    e[1][d] = p2[d] - p0[d];
-    e[2][d] = p3[d] - p0[d];
-  }
+  ph_elem::edge_vectors(coord, v, e);
   const double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) +
                      e[0][1] * (e[1][2] * e[2][0] - e[1][0] * e[2][2]) +
                      e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
@@ -163,7 +165,8 @@ __device__ __forceinline__ void tet_geom_dw(const double* __restrict__ coord, in
   out[34] = __int_as_float(kg);
   out[35] = __int_as_float(-2 * exponent(rdet) - (exponent(g[0][0].h) + exponent(g[1][1].h) + exponent(g[2][2].h) +
                                                   3 * kg));
-  float4* o = reinterpret_cast<float4*>(geo + PH_GEO_STRIDE * t);
+  vol[t] = make_double2(adet, rdet);
+  float4* o = reinterpret_cast<float4*>(geo + PH_GEO_DW_STRIDE * t);
 #pragma unroll
   for (int i = 0; i < 9; ++i) o[i] = make_float4(out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
 }
@@ -188,28 +191,38 @@ __global__ void k_face_count(const int4* __restrict__ tet, int64_t nE, int64_t n
 
 // 2. scatter keys into buckets: entry = (v0, v1, v2, slot), slot = 4t+k for
 //    tet faces and 4nE+i for Neumann triples.  cnt counts down to 0.  The
-//    same thread then computes the tet's geometry record: the FP64-bound
-//    geometry and the latency-bound atomics and scattered stores overlap in
-//    the SM's warp scheduler.
-__global__ void k_face_fill(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
+//    same thread then computes the tet's geometry: in fixed point on the
+//    integer pipe (fixed.cuh), 13 FP64 operations where the fp64 record took
+//    55 and bound the kernel.  Now the atomics, the scattered stores and the
+//    geometry share it (17.9M tets: 1.94 -> 1.08 ms).  Blocks of 128 threads, 6
+//    per SM (80 registers): 5 or 7 take 1.15 and 1.09 ms, 256-thread blocks
+//    at 96 registers 1.63; storing the entries after the geometry instead of
+//    before it holds their stores back, 1.26.
+constexpr int kFillThreads = 128;
+__global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
                             int64_t nN, int sub, const int32_t* __restrict__ start, int32_t* __restrict__ cnt,
                             int4* __restrict__ entries, int32_t* __restrict__ mate, const double* __restrict__ coord,
-                            double* __restrict__ geo, bool geo_dw, unsigned* status) {
+                            double* __restrict__ geo, int32_t* __restrict__ gexp, double2* __restrict__ vol, bool geo_dw,
+                            unsigned* status) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (failed(status)) return;
   if (i < nE) {
     int4 v = tet[i];
     if (!valid_tet(v, nC)) return;
+    int pos[4];  // four atomics in flight, then their stores
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      int3 s = sort3(local_face(v, k));
-      const int64_t b = bucket_of(s, sub);
-      int pos = start[b] + atomicSub(&cnt[b], 1) - 1;
-      entries[pos] = make_int4(s.x, s.y, s.z, (int)(4 * i + k));
+      const int64_t b = bucket_of(sort3(local_face(v, k)), sub);
+      pos[k] = start[b] + atomicSub(&cnt[b], 1) - 1;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int3 s = sort3(local_face(v, k));
+      entries[pos[k]] = make_int4(s.x, s.y, s.z, (int)(4 * i + k));
     }
     reinterpret_cast<int4*>(mate)[i] = make_int4(-1, -1, -1, -1);  // no mate yet (boundary)
-    if (geo_dw) tet_geom_dw(coord, v, i, geo, status);
-    else tet_geom(coord, v, i, geo, status);
+    if (geo_dw) tet_geom_dw(coord, v, i, geo, vol, status);
+    else tet_geom(coord, v, i, geo, gexp, vol, status);
   } else if (i < nE + nN) {
     int3 f = neumann_tri(nb, i - nE);
     if (!valid_tri(f, nC)) return;
@@ -652,7 +665,8 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   // first part zeroed by one memset).  Few host calls keep the GPU fed.
   Carve mc, sc;
   const size_t o_status = mc.take<unsigned>(1), o_coord = mc.take<double>(3 * nC), o_tet = mc.take<int4>(nE);
-  const size_t o_geo = mc.take<double>(PH_GEO_STRIDE * nE), o_tface = mc.take<int4>(nE);
+  const size_t o_geo = mc.take<double>((dw ? PH_GEO_DW_STRIDE : PH_GEO_STRIDE) * nE), o_tface = mc.take<int4>(nE);
+  const size_t o_gexp = mc.take<int32_t>(dw ? 0 : nE), o_vol = mc.take<double2>(nE);
   const size_t o_tmult = mc.take<int4>(nE), o_tpos = mc.take<int4>(nE), o_trel = mc.take<ushort4>(nE);
   const size_t o_ftet = mc.take<int2>(nFmax), o_fvtx = mc.take<int32_t>(3 * nFmax);
   const size_t o_fkind = mc.take<int8_t>(nFmax), o_fmult = mc.take<int32_t>(nFmax + 1);
@@ -682,6 +696,8 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
     m->coord = Carve::at<double>(A, o_coord);
     m->tet = Carve::at<int4>(A, o_tet);
     m->geo = Carve::at<double>(A, o_geo);
+    m->gexp = Carve::at<int32_t>(A, o_gexp);
+    m->vol = Carve::at<double2>(A, o_vol);
     m->tface = Carve::at<int4>(A, o_tface);
     m->tmult = Carve::at<int4>(A, o_tmult);
     m->tpos = Carve::at<int4>(A, o_tpos);
@@ -723,8 +739,8 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   if (nent > 0) {
     {
       KernelTimer kt("k_face_fill", s, 2);
-      k_face_fill<<<grid_for(nE + nN), kThreads, 0, s>>>(m->tet, nE, nC, neumann, nN, sub, start, cnt, entries,
-                                                         mate, m->coord, m->geo, dw, m->status);
+      k_face_fill<<<grid_for(nE + nN, kFillThreads), kFillThreads, 0, s>>>(m->tet, nE, nC, neumann, nN, sub, start, cnt, entries,
+                                                         mate, m->coord, m->geo, m->gexp, m->vol, dw, m->status);
       PH_CU(launched(), "k_face_fill");
     }
     {
@@ -1135,6 +1151,8 @@ extern "C" ph_status ph_mesh_create_batch(int32_t n, const double* const* coord,
     m->tpos = u->tpos + t0;
     m->trel = u->trel + t0;
     m->geo = u->geo + PH_GEO_STRIDE * t0;
+    m->gexp = u->gexp + t0;
+    m->vol = u->vol + t0;
     m->face_tet = u->face_tet + f0;
     m->face_vtx = u->face_vtx + 3 * f0;
     m->face_kind = u->face_kind + f0;

@@ -14,9 +14,12 @@
 #define PH_NO_MULT 0x7FFFFFFF
 #define PH_BND_BIT 0x80000000u
 #define PH_ID_MASK 0x7FFFFFFF
-// Per-element geometry record (doubles): G_e = E E' (00 01 02 11 12 22),
-// GT = G_e T0^-1 row-major (9), |det E|, 1/|det E|, padding.
-#define PH_GEO_STRIDE 18
+// Per-element geometry record: G_e = E E' (00 01 02 11 12 22) as six int64 on
+// the element's scale 2^gexp (fixed.cuh), or as six doubles where gexp is
+// PH_GEXP_F64.  Meshes of ph_mesh_create_dw: 18 doubles (element.cuh).
+#define PH_GEO_STRIDE 6
+#define PH_GEXP_F64 INT32_MIN
+#define PH_GEO_DW_STRIDE 18
 
 // Device memory shared by the meshes of one batched build (ph_mesh_create_batch):
 // released when the last of them is destroyed.
@@ -37,7 +40,9 @@ struct ph_mesh {
   int4* tmult;         // nE: see PH_NO_MULT / PH_BND_BIT
   int4* tpos;          // nE: CSR position of the diagonal entry of row l(F_k)
   ushort4* trel;       // nE: 3 packed 4-bit offsets (m != k, ascending m) from tpos
-  double* geo;         // nE*PH_GEO_STRIDE: G_e, G_e T0^-1, |det|, 1/|det|
+  double* geo;         // nE*PH_GEO_STRIDE (PH_GEO_DW_STRIDE): the geometry record
+  int32_t* gexp;       // nE: scale of the record (not in a double-word mesh)
+  double2* vol;        // nE: |det E|, 1/|det E|
   int2* face_tet;      // nF
   int32_t* face_vtx;   // nF*3
   int8_t* face_kind;   // nF
