@@ -126,16 +126,11 @@ ph_status ph_mesh_create_batch(int32_t n, const double* const* coord, const int6
                                ph_mesh** out);
 
 /*
- * ph_mesh_create for the double-word path (a precision variant; the paper has
- * no counterpart): the same connectivity, numbering and CSR pattern, bit for
- * bit, but the per-element geometry record holds G_e and G_e T0^-1 as scaled
- * pairs of floats, computed in double-word arithmetic on the FP32 pipe from
- * the fp64 edge vectors (|det E|, 1/|det E| and the face areas |F| stay the
- * fp64 values: the leading terms of H and of the recovery need their last
- * bits).  Such a mesh works with ph_assemble_dw, ph_recover_factored(_dw), ph_misfit,
- * ph_adjoint_rhs and every connectivity, CSR and solver entry point; the
- * entry points that read the fp64 record (ph_assemble, ph_recover,
- * ph_adjoint_grad, ph_batch_create) return PH_ERR_ARG for it.
+ * ph_mesh_create for the double-word entry points (a precision variant; the
+ * paper has no counterpart): the same mesh, bit for bit.  It works with
+ * ph_assemble_dw, ph_recover_factored(_dw), ph_misfit, ph_adjoint_rhs and every
+ * connectivity, CSR and solver entry point; ph_assemble, ph_recover,
+ * ph_adjoint_grad and ph_batch_create return PH_ERR_ARG for it.
  */
 ph_status ph_mesh_create_dw(const double* coord, int64_t nC, const int32_t* tet, int64_t nE,
                             const int32_t* neumann, int64_t nN, void* stream, ph_mesh** out);
@@ -200,16 +195,10 @@ ph_status ph_assemble(const ph_mesh* mesh, const double* a, double c, const doub
                       double* factor, void* stream);
 
 /*
- * ph_assemble with the element condensation kernel (the 3x3 algebra behind
- * A(T)^-1 on the complement of the constants, Eq. schur) evaluated in
- * double-word arithmetic on the FP32 pipe: pairs of floats carrying ~48
- * significant bits (Dekker's exact transforms; the error bounds of Joldes,
- * Muller and Popescu 2017), with the leading term d d'/(c|T|), |det|, |F|
- * and every sum of H and rhs kept in fp64.  A precision variant, not in the
- * paper: same arguments, outputs and error behaviour as ph_assemble, results
- * within ~1e-14 relative of it (both within 1e-12 of the exact values).  An
- * element whose reaction term dominates (c h^2 comparable to a) or whose
- * data leave the exponent range of the float pairs is condensed in fp64.
+ * ph_assemble for either kind of mesh: same arguments, outputs and error
+ * behaviour, and the same bits.  (The variant once ran the condensation kernel
+ * in pairs of floats of ~48 significant bits; the fixed-point kernel of
+ * ph_assemble is faster than that and as accurate as fp64, so it serves both.)
  */
 ph_status ph_assemble_dw(const ph_mesh* mesh, const double* a, double c, const double* f_face,
                          const double* uD_face, const double* gN_face, double* values, double* rhs, double* factor,
@@ -301,8 +290,7 @@ ph_status ph_solve_pcg_noalloc(int64_t n, const int32_t* rowptr, const int32_t* 
 /*
  * Batched assembly (not in the paper): many problems, meshes of uneven size
  * each with its own coefficient field, assembled and condensed by one
- * persistent kernel (plus one kernel that clears the entries receiving atomic
- * contributions).  Each problem's values, rhs and factor are bit-identical to
+ * persistent kernel (plus one kernel that clears values and rhs first).  Each problem's values, rhs and factor are bit-identical to
  * a plain ph_assemble call on it.  A batch is not thread-safe.
  *   ph_batch_create   group n meshes (the meshes must outlive the batch).
  *   ph_batch_bind     per-problem arrays: host arrays of n DEVICE pointers

@@ -42,8 +42,8 @@ namespace {
 // tets: 3.70 -> 2.31 ms; the FP64 pipe alone needs 1.9).  Six blocks of 128
 // threads per SM (80 registers): 4 (122 registers), 5 and 7 take 2.70, 2.40
 // and 2.31 ms.
-template <bool UD, bool GN, bool FAC, bool DW>
-__global__ void __launch_bounds__(128, DW ? 7 : 6) k_assemble(int64_t nE, const double* __restrict__ geo,
+template <bool UD, bool GN, bool FAC>
+__global__ void __launch_bounds__(128, 6) k_assemble(int64_t nE, const double* __restrict__ geo,
                                                   const int32_t* __restrict__ gexp, const double2* __restrict__ vol,
                                                   const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                   const int4* __restrict__ tpos, const ushort4* __restrict__ trel,
@@ -51,12 +51,11 @@ __global__ void __launch_bounds__(128, DW ? 7 : 6) k_assemble(int64_t nE, const 
                                                   double c20, double six_over_c, const double* __restrict__ f_face,
                                                   const double* __restrict__ uD, const double* __restrict__ gN,
                                                   double* __restrict__ values, double* __restrict__ rhs,
-                                                  double* __restrict__ factor, unsigned* status,
-                                                  const double* __restrict__ coord, const int4* __restrict__ tet) {
+                                                  double* __restrict__ factor, unsigned* status) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
-  assemble_element<UD, GN, FAC, DW>(t, geo, gexp, vol, tface, tmult, tpos, trel, face_area, a, c20, six_over_c, f_face, uD,
-                                      gN, values, rhs, factor, status, coord, tet);
+  assemble_element(UD, GN, FAC, t, geo, gexp, vol, tface, tmult, tpos, trel, face_area, a, c20, six_over_c, f_face, uD,
+                                gN, values, rhs, factor, status);
 }
 
 
@@ -114,24 +113,23 @@ bool finite_pos(double x) { return x > 0.0 && x < INFINITY; }
 
 using namespace ph;
 
-// The fp64 entry points need the fp64 geometry record, which a mesh from
-// ph_mesh_create_dw does not hold.
+// A mesh from ph_mesh_create_dw is for the double-word entry points: the fp64
+// ones refuse it.
 static bool needs_fp64_record(const ph_mesh* m, const char* who) {
   if (!m->geo_dw) return false;
   char msg[160];
-  snprintf(msg, sizeof msg, "%s: the mesh holds a double-word geometry record (ph_mesh_create_dw)", who);
+  snprintf(msg, sizeof msg, "%s: the mesh is for the double-word entry points (ph_mesh_create_dw)", who);
   set_error_text(msg);
   return true;
 }
 
-template <bool DW>
 static void launch_assemble(const ph_mesh* m, unsigned grid, bool ud, bool gn, double c20, double six_over_c,
                             const double* a, const double* f_face, const double* uD_face, const double* gN_face,
                             double* values, double* rhs, double* factor, cudaStream_t s) {
 #define PH_ASM(UDV, GNV, FACV)                                                                                  \
-  k_assemble<UDV, GNV, FACV, DW><<<grid, 128, 0, s>>>(m->nE, m->geo, m->gexp, m->vol, m->tface, m->tmult,       \
+  k_assemble<UDV, GNV, FACV><<<grid, 128, 0, s>>>(m->nE, m->geo, m->gexp, m->vol, m->tface, m->tmult,       \
                                                       m->tpos, m->trel, m->face_area, a, c20, six_over_c, f_face, uD_face,     \
-                                                        gN_face, values, rhs, factor, m->status, m->coord, m->tet)
+                                                        gN_face, values, rhs, factor, m->status)
   if (factor) {
     if (ud && gn) PH_ASM(true, true, true);
     else if (ud) PH_ASM(true, false, true);
@@ -170,10 +168,7 @@ static ph_status assemble(const ph_mesh* m, const double* a, double c, const dou
   const unsigned grid = grid_for(m->nE, 128);
   const bool ud = uD_face != nullptr && m->nFd > 0, gn = gN_face != nullptr && m->nFn > 0;
   KernelTimer kt(DW ? "k_assemble_dw" : "k_assemble", s);
-  if (m->geo_dw)
-    launch_assemble<true>(m, grid, ud, gn, c20, six_over_c, a, f_face, uD_face, gN_face, values, rhs, factor, s);
-  else
-    launch_assemble<false>(m, grid, ud, gn, c20, six_over_c, a, f_face, uD_face, gN_face, values, rhs, factor, s);
+  launch_assemble(m, grid, ud, gn, c20, six_over_c, a, f_face, uD_face, gN_face, values, rhs, factor, s);
   const cudaError_t e = launched();
   kt.stop();
   return cuda_status(e, "k_assemble");

@@ -6,8 +6,8 @@
 // (blocks per SM x SMs) blocks walks the tile table round-robin; each block
 // runs the plain path's per-element code (assemble_element) on the tile's
 // elements, so every problem's values, rhs and factor are bit-identical to a
-// plain ph_assemble call.  The entries that receive atomic contributions are
-// cleared first by one batched zero kernel.  The tile size and block shape come
+// plain ph_assemble call.  Values and rhs are cleared first by one batched zero
+// kernel.  The tile size and block shape come
 // from ph_batch_autotune, which times candidate configurations on the bound
 // problems; the two launches can be instantiated once as a CUDA graph.
 #include <math.h>
@@ -23,7 +23,7 @@ using namespace ph_elem;
 
 namespace {
 
-struct ProbDesc {
+struct alignas(8) ProbDesc {
   const double* geo;
   const int32_t* gexp;
   const double2* vol;
@@ -32,8 +32,7 @@ struct ProbDesc {
   const int4* tpos;
   const ushort4* trel;
   const double* area;
-  const int32_t* rowdiag;
-  int64_t nE, L;
+  int64_t nE, L, nnz;
   const double* a;
   const double* f;
   const double* uD;
@@ -55,27 +54,31 @@ struct Tile {
   int64_t start;
 };
 
-template <bool UD, bool GN, bool FAC>
-__device__ __forceinline__ void run_tile(const ProbDesc& d, int64_t start, int count) {
-  for (int i = threadIdx.x; i < count; i += blockDim.x)
-    assemble_element<UD, GN, FAC>(start + i, d.geo, d.gexp, d.vol, d.tface, d.tmult, d.tpos, d.trel, d.area, d.a, d.c20,
-                                  d.six_over_c, d.f, d.uD, d.gN, d.values, d.rhs, d.factor, d.status);
-}
-
-// persistent: block b takes tiles b, b + gridDim.x, ...
-__global__ void k_batch_assemble(const ProbDesc* __restrict__ probs, const Tile* __restrict__ tiles, int64_t ntiles) {
+// persistent: block b takes tiles b, b + gridDim.x, ...  The problem's descriptor
+// sits in shared memory and is read again for every element: in registers its
+// 20 fields, with a copy of the element code for each of the eight flag
+// combinations, took 164 of them and left 12 warps on an SM, enough while the
+// FP64 pipe bound the kernel.  MAXT threads at most per block.
+template <int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) k_batch_assemble(const ProbDesc* __restrict__ probs,
+                                                               const Tile* __restrict__ tiles, int64_t ntiles) {
+  __shared__ ProbDesc d;
+  int have = -1;
   for (int64_t k = blockIdx.x; k < ntiles; k += gridDim.x) {
     const Tile tl = tiles[k];
-    const ProbDesc& d = probs[tl.prob];
-    switch (d.flags) {  // uniform across the block
-      case 0: run_tile<false, false, false>(d, tl.start, tl.count); break;
-      case 1: run_tile<true, false, false>(d, tl.start, tl.count); break;
-      case 2: run_tile<false, true, false>(d, tl.start, tl.count); break;
-      case 3: run_tile<true, true, false>(d, tl.start, tl.count); break;
-      case 4: run_tile<false, false, true>(d, tl.start, tl.count); break;
-      case 5: run_tile<true, false, true>(d, tl.start, tl.count); break;
-      case 6: run_tile<false, true, true>(d, tl.start, tl.count); break;
-      default: run_tile<true, true, true>(d, tl.start, tl.count); break;
+    if (tl.prob != have) {  // uniform across the block
+      __syncthreads();
+      for (unsigned i = threadIdx.x; i < sizeof(ProbDesc) / 8; i += blockDim.x)
+        reinterpret_cast<unsigned long long*>(&d)[i] = reinterpret_cast<const unsigned long long*>(probs + tl.prob)[i];
+      __syncthreads();
+      have = tl.prob;
+    }
+#pragma unroll 1
+    for (int i = threadIdx.x; i < tl.count; i += blockDim.x) {
+      asm volatile("" ::: "memory");
+      assemble_element(d.flags & 1, d.flags & 2, d.flags & 4, tl.start + i, d.geo, d.gexp, d.vol, d.tface, d.tmult,
+                       d.tpos, d.trel, d.area, d.a, d.c20, d.six_over_c, d.f, d.uD, d.gN, d.values, d.rhs, d.factor,
+                       d.status);
     }
   }
 }
@@ -98,20 +101,30 @@ __global__ void k_batch_recover(const ProbDesc* __restrict__ probs, const Tile* 
   }
 }
 
-// rhs = 0 and the diagonal of every row = 0, for all problems (row offsets
-// of the problems are the exclusive prefix sums roff)
-__global__ void k_batch_zero(const ProbDesc* __restrict__ probs, const int64_t* __restrict__ roff, int32_t nprob,
-                             int64_t nrows) {
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < nrows; g += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = nprob - 1;  // problem of row g: last roff[p] <= g
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (roff[mid] <= g) lo = mid; else hi = mid - 1;
-    }
-    const ProbDesc& d = probs[lo];
-    const int64_t l = g - roff[lo];
-    d.rhs[l] = 0.0;
-    d.values[d.rowdiag[l]] = 0.0;
+// Zeros in entries [lo, hi) of x, 16 bytes at a time where x is aligned.
+__device__ __forceinline__ void zero_range(double* __restrict__ x, int64_t lo, int64_t hi) {
+  double* p = x + lo;
+  int64_t n = hi - lo;
+  if (n > 0 && (reinterpret_cast<uintptr_t>(p) & 15)) {
+    if (threadIdx.x == 0) *p = 0.0;
+    ++p;
+    --n;
+  }
+  for (int64_t i = threadIdx.x; i < n / 2; i += blockDim.x) reinterpret_cast<double2*>(p)[i] = make_double2(0.0, 0.0);
+  if ((n & 1) && threadIdx.x == 0) p[n - 1] = 0.0;
+}
+
+// values = 0 and rhs = 0 for all problems: tile [start, start + count) of a
+// problem's elements takes the same share of its entries.  Whole arrays, as in
+// ph_assemble: stores to the diagonal positions alone make L2 read every sector
+// of the array first (75M rows: 0.98 ms against 0.66).
+__global__ void k_batch_zero(const ProbDesc* __restrict__ probs, const Tile* __restrict__ tiles, int64_t ntiles) {
+  for (int64_t k = blockIdx.x; k < ntiles; k += gridDim.x) {
+    const Tile tl = tiles[k];
+    const ProbDesc& d = probs[tl.prob];
+    const int64_t s = tl.start, e = tl.start + tl.count;
+    zero_range(d.values, d.nnz * s / d.nE, d.nnz * e / d.nE);
+    zero_range(d.rhs, d.L * s / d.nE, d.L * e / d.nE);
   }
 }
 
@@ -123,8 +136,7 @@ struct ph_batch {
   std::vector<const ph_mesh*> meshes;
   std::vector<ProbDesc> host;
   ProbDesc* d_probs;
-  int64_t* d_roff;
-  int64_t nrows, nelems;
+  int64_t nelems;
   Tile* d_tiles;
   int64_t ntiles;
   int32_t tile, threads, blocks_per_sm, sms;
@@ -166,8 +178,8 @@ extern "C" ph_status ph_batch_create(ph_mesh* const* meshes, int32_t n, void* st
   *out = nullptr;
   for (int32_t i = 0; i < n; ++i) {
     if (!meshes[i]) return PH_ERR_ARG;
-    if (meshes[i]->geo_dw) {  // the batched kernel runs the fp64 element code
-      set_error_text("ph_batch_create: a mesh holds a double-word geometry record (ph_mesh_create_dw)");
+    if (meshes[i]->geo_dw) {
+      set_error_text("ph_batch_create: a mesh is for the double-word entry points (ph_mesh_create_dw)");
       return PH_ERR_ARG;
     }
   }
@@ -177,34 +189,28 @@ extern "C" ph_status ph_batch_create(ph_mesh* const* meshes, int32_t n, void* st
   b->meshes.assign(meshes, meshes + n);
   b->host.resize(n);
   b->d_probs = nullptr;
-  b->d_roff = nullptr;
   b->d_tiles = nullptr;
   b->graph = nullptr;
   b->exec = nullptr;
   b->bound = false;
   b->recover = false;
+  // 256 problems, 37.2M tets, assembly and recovery: 9.2 ms; 128 x 4 9.7, 256 x 3
+  // 9.4, 256 x 8 9.6 (more blocks than fit even out the tiles' ends)
   b->tile = 1024;
-  b->threads = 128;
-  b->blocks_per_sm = 4;
+  b->threads = 256;
+  b->blocks_per_sm = 6;
   cudaError_t e = cudaGetDevice(&b->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
-  std::vector<int64_t> roff(n + 1, 0);
   b->nelems = 0;
   for (int32_t i = 0; i < n; ++i) {
-    roff[i + 1] = roff[i] + meshes[i]->L;
     b->nelems += meshes[i]->nE;
     if (meshes[i]->device != b->device) e = cudaErrorInvalidDevice;
   }
-  b->nrows = roff[n];
   if (e == cudaSuccess) e = alloc(&b->d_probs, (size_t)std::max(n, 1), s);
-  if (e == cudaSuccess) e = alloc(&b->d_roff, (size_t)n + 1, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_roff, roff.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   ph_status st = cuda_status(e, "ph_batch_create");
   if (st == PH_OK) st = build_tiles(b, s);
   if (st != PH_OK) {
     free_async(b->d_probs, s);
-    free_async(b->d_roff, s);
     free_async(b->d_tiles, s);
     delete b;
     return st;
@@ -218,7 +224,6 @@ extern "C" ph_status ph_batch_destroy(ph_batch* b, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   drop_graph(b);
   free_async(b->d_probs, s);
-  free_async(b->d_roff, s);
   free_async(b->d_tiles, s);
   delete b;
   return PH_OK;
@@ -252,8 +257,8 @@ extern "C" ph_status ph_batch_bind(ph_batch* b, const double* const* a, const do
     d.tpos = m->tpos;
     d.trel = m->trel;
     d.area = m->face_area;
-    d.rowdiag = m->rowdiag;
     d.nE = m->nE;
+    d.nnz = m->nnz;
     d.L = m->L;
     d.a = a[i];
     d.f = f_face[i];
@@ -277,15 +282,16 @@ extern "C" ph_status ph_batch_bind(ph_batch* b, const double* const* a, const do
 }
 
 static cudaError_t launch_batch(ph_batch* b, cudaStream_t s) {
-  if (b->nrows > 0) {
-    const unsigned zg = (unsigned)std::min<int64_t>((b->nrows + 255) / 256, (int64_t)b->sms * 8);
-    k_batch_zero<<<zg, 256, 0, s>>>(b->d_probs, b->d_roff, b->n, b->nrows);
+  if (b->ntiles > 0) {
+    const unsigned zg = (unsigned)std::min<int64_t>(b->ntiles, (int64_t)b->sms * 8);
+    k_batch_zero<<<zg, 256, 0, s>>>(b->d_probs, b->d_tiles, b->ntiles);
     cudaError_t e = launched();
     if (e != cudaSuccess) return e;
   }
   if (b->ntiles > 0) {
     const unsigned grid = (unsigned)std::min<int64_t>(b->ntiles, (int64_t)b->sms * b->blocks_per_sm);
-    k_batch_assemble<<<grid, b->threads, 0, s>>>(b->d_probs, b->d_tiles, b->ntiles);
+    if (b->threads <= 256) k_batch_assemble<256, 3><<<grid, b->threads, 0, s>>>(b->d_probs, b->d_tiles, b->ntiles);
+    else k_batch_assemble<1024, 1><<<grid, b->threads, 0, s>>>(b->d_probs, b->d_tiles, b->ntiles);
     cudaError_t e = launched();
     if (e != cudaSuccess || !b->recover) return e;
     k_batch_recover<<<grid, b->threads, 0, s>>>(b->d_probs, b->d_tiles, b->ntiles);
@@ -295,7 +301,7 @@ static cudaError_t launch_batch(ph_batch* b, cudaStream_t s) {
 }
 
 static int batch_launches(const ph_batch* b) {
-  return (b->nrows > 0 ? 1 : 0) + (b->ntiles > 0 ? (b->recover ? 2 : 1) : 0);
+  return b->ntiles > 0 ? (b->recover ? 3 : 2) : 0;
 }
 
 extern "C" ph_status ph_batch_assemble(ph_batch* b, void* stream) {

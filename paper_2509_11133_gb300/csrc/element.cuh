@@ -39,8 +39,7 @@ __device__ __forceinline__ void edge_vectors(const double* __restrict__ coord, i
 }
 
 // Element geometry in fp64: G_e = E E', |det E| and 1/|det E| (the Newton
-// reciprocal), for the elements that fx::geometry leaves to fp64 and those the
-// double-word kernel hands to the fp64 path.
+// reciprocal), for the elements that fx::geometry leaves to fp64.
 __device__ __forceinline__ Geo compute_geo(const double e[3][3]) {
   const double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) +
                      e[0][1] * (e[1][2] * e[2][0] - e[1][0] * e[2][2]) +
@@ -125,129 +124,14 @@ __device__ __forceinline__ void element_kernel(const Record& r, double2 vol, dou
     face_kernel(to_f64(r, vol), a, c20, 6.0 / 9.0, Q);
 }
 
-// The geometry of one element in double-word form: G' = 2^-kg G_e and
-// G'T = 2^-kg G_e T0^-1, 2^kg the binade of the largest diagonal entry of
-// G_e (so every value is below ~8 in magnitude), |det E| and 1/|det E| in
-// fp64, and the binade of |det E|^2 / (g00 g11 g22) (the element's
-// flatness, within a factor 16).
-struct GeoDW {
-  dw::f2 g[6];  // G' 00 01 02 11 12 22
-  dw::f2 t[9];  // G'T row-major
-  double adet, rdet;
-  int kg, flat;
-};
-
-// The double-word record of a mesh built by ph_mesh_create_dw (144 bytes per
-// element: 30 floats of pairs, then |det E| and
-// 1/|det E| as doubles 15 and 16, then kg and the flatness as two ints).
-__device__ __forceinline__ GeoDW load_geo_dw(const double* __restrict__ geo, int64_t t) {
-  const float4* p = reinterpret_cast<const float4*>(geo + PH_GEO_DW_STRIDE * t);
-  float v[36];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const float4 q = __ldg(p + i);
-    v[4 * i] = q.x;
-    v[4 * i + 1] = q.y;
-    v[4 * i + 2] = q.z;
-    v[4 * i + 3] = q.w;
-  }
-  GeoDW D;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) D.g[i] = dw::f2{v[2 * i], v[2 * i + 1]};
-#pragma unroll
-  for (int i = 0; i < 9; ++i) D.t[i] = dw::f2{v[12 + 2 * i], v[13 + 2 * i]};
-  D.adet = __hiloint2double(__float_as_int(v[31]), __float_as_int(v[30]));
-  D.rdet = __hiloint2double(__float_as_int(v[33]), __float_as_int(v[32]));
-  D.kg = __float_as_int(v[34]);
-  D.flat = __float_as_int(v[35]);
-  return D;
-}
-
-// The same Qf (times sc = sc6/6) with the 3x3 algebra in double-word
-// arithmetic on the FP32 pipe (dw.cuh), for the assembly variant of
-// ph_assemble_dw.  The element is first made dimensionless with exact powers
-// of two: G_e and G_e T0^-1 are scaled by 2^-k, 2^k the largest diagonal
-// entry's binade, so that
-//     Qv = 6 / (a |det E|) 2^k D0' (T0 + gamma G')^-1 G'T D0,
-//     G' = 2^-k G_e, G'T = 2^-k G_e T0^-1, gamma = c 2^k / (20 a),
-// and the double-word values stay within a few binades of 1; the scalar's
-// power of two goes into the conversion back to fp64.  The path is taken when
-// gamma G' is small against T0 (gamma 2^-k max g_ii <= 2^-2: the 3x3 matrix
-// then has condition number <= 6 and the double-word result is accurate to
-// ~1e-14 relative) and the element is not flat (|det E|^2 >= 2^-12 g00 g11
-// g22, judged on the exponents: the Kuhn elements and their refinements
-// sit near 2^-3, the jittered ones above 2^-10; on flatter elements the
-// condensation kernel's cancellations would cost the float pairs' 5 bits
-// fewer than fp64 more than the 1e-12 the results are held to).  Otherwise
-// -- a reaction term that dominates the element (c h^2 > a), a flat element,
-// or inputs beyond the exponent range -- it returns false and the caller
-// takes the fp64 path.
-__device__ __forceinline__ bool face_kernel_dw(const GeoDW& D, double a, double c20, double sc6, double Q[10]) {
-  using namespace dw;
-  const int kg = D.kg;
-  const int ka = exponent(a), kc = exponent(c20), kr = exponent(D.rdet);
-  const int p = kc + kg - ka;  // binade of gamma (within a factor 4)
-  const int K = kr - ka + kg;  // binade of the overall scalar 6/(a |det E|) 2^k (with sc)
-  if (p > -4 || D.flat < -12 || kg < -900 || kg > 900 || ka < -900 || ka > 900 || K < -900 || K > 900) return false;
-  const f2 am = from_double(a, -ka), cm = from_double(c20, -kc);  // mantissas in [1, 2)
-  const f2 ra = rcp(am);
-  // gamma G' and the 3x3 matrix T0 + gamma G' (T0 = I + 1 1')
-  f2 m00, m01, m02, m11, m12, m22;
-  if (p < -100) {  // gamma G' below 2^-98 of T0: T0 alone
-    m00 = m11 = m22 = f2{2.f, 0.f};
-    m01 = m02 = m12 = f2{1.f, 0.f};
-  } else {
-    const f2 gam = ldexp(mul(cm, ra), p);
-    m00 = add(mul(gam, D.g[0]), 2.f);
-    m01 = add(mul(gam, D.g[1]), 1.f);
-    m02 = add(mul(gam, D.g[2]), 1.f);
-    m11 = add(mul(gam, D.g[3]), 2.f);
-    m12 = add(mul(gam, D.g[4]), 1.f);
-    m22 = add(mul(gam, D.g[5]), 2.f);
-  }
-  // adjugate and determinant
-  const f2 A00 = sub(mul(m11, m22), mul(m12, m12));
-  const f2 A01 = sub(mul(m02, m12), mul(m01, m22));
-  const f2 A02 = sub(mul(m01, m12), mul(m02, m11));
-  const f2 A11 = sub(mul(m00, m22), mul(m02, m02));
-  const f2 A12 = sub(mul(m01, m02), mul(m00, m12));
-  const f2 A22 = sub(mul(m00, m11), mul(m01, m01));
-  const f2 det = add(add(mul(m00, A00), mul(m01, A01)), mul(m02, A02));
-  // scalar: sc 6/(a |det E|) / det M' with its power of two 2^K kept apart
-  const f2 sc = mul(mul(mul(from_double(sc6), from_double(D.rdet, -kr)), ra), rcp(det));
-  const f2* t = D.t;
-  // Y = adj(M') G'T (symmetric), scaled
-  const f2 y00 = mul(add(add(mul(A00, t[0]), mul(A01, t[3])), mul(A02, t[6])), sc);
-  const f2 y01 = mul(add(add(mul(A00, t[1]), mul(A01, t[4])), mul(A02, t[7])), sc);
-  const f2 y02 = mul(add(add(mul(A00, t[2]), mul(A01, t[5])), mul(A02, t[8])), sc);
-  const f2 y11 = mul(add(add(mul(A01, t[1]), mul(A11, t[4])), mul(A12, t[7])), sc);
-  const f2 y12 = mul(add(add(mul(A01, t[2]), mul(A11, t[5])), mul(A12, t[8])), sc);
-  const f2 y22 = mul(add(add(mul(A02, t[2]), mul(A12, t[5])), mul(A22, t[8])), sc);
-  // Qv = D0' Y D0; faces 0,1,2,3 sit opposite vertices 3,1,2,0
-  const f2 c0 = add(add(y00, y01), y02), c1 = add(add(y01, y11), y12), c2 = add(add(y02, y12), y22);
-  Q[ut(0, 0)] = to_double(y22, K);
-  Q[ut(0, 1)] = to_double(y02, K);
-  Q[ut(0, 2)] = to_double(y12, K);
-  Q[ut(0, 3)] = to_double(neg(c2), K);
-  Q[ut(1, 1)] = to_double(y00, K);
-  Q[ut(1, 2)] = to_double(y01, K);
-  Q[ut(1, 3)] = to_double(neg(c0), K);
-  Q[ut(2, 2)] = to_double(y11, K);
-  Q[ut(2, 3)] = to_double(neg(c1), K);
-  Q[ut(3, 3)] = to_double(add(add(c0, c1), c2), K);
-  return true;
-}
-
 using ph::neg_if;
 
 
 // Local matrices, condensation and scatter of element t (Section 4.2-4.3,
 // Eq. schur): the body of the assembly kernels (one thread per element).
-// DW: the double-word record of a mesh from ph_mesh_create_dw (elements the
-// double-word kernel hands back get their fp64 geometry recomputed from coord
-// and tet); else the fixed-point record.
-template <bool UD, bool GN, bool FAC, bool DW = false>
-__device__ __forceinline__ void assemble_element(int64_t t, const double* __restrict__ geo,
+// UD, GN, FAC: u_D and g_N given, the factor wanted (constants of the plain
+// kernels, the problem's in the batched one).
+__device__ __forceinline__ void assemble_element(bool UD, bool GN, bool FAC, int64_t t, const double* __restrict__ geo,
                                                  const int32_t* __restrict__ gexp, const double2* __restrict__ vol,
                                                  const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                  const int4* __restrict__ tpos, const ushort4* __restrict__ trel,
@@ -255,19 +139,14 @@ __device__ __forceinline__ void assemble_element(int64_t t, const double* __rest
                                                  double c20, double six_over_c, const double* __restrict__ f_face,
                                                  const double* __restrict__ uD, const double* __restrict__ gN,
                                                  double* __restrict__ values, double* __restrict__ rhs,
-                                                 double* __restrict__ factor, unsigned* status,
-                                                 const double* __restrict__ coord = nullptr,
-                                                 const int4* __restrict__ tet = nullptr) {
+                                                 double* __restrict__ factor, unsigned* status) {
   const double at = __ldg(a + t);
   if (!ph::pos_finite(at)) {
     ph_flag(status, PH_ERR_ARG);
     return;
   }
   const double2 vt = __ldg(vol + t);  // |det E|, 1/|det E|
-  Record R;
-  GeoDW D;
-  if (DW) D = load_geo_dw(geo, t);
-  else R = load_record(geo, gexp, t);
+  const Record R = load_record(geo, gexp, t);
   const int4 tf = __ldg(tface + t);
   const int4 tm = __ldg(tmult + t);
   int F[4];
@@ -286,13 +165,7 @@ __device__ __forceinline__ void assemble_element(int64_t t, const double* __rest
     if (GN && comp(tm, k) == PH_NO_MULT) h[k] = fma(ar[k], __ldg(gN + F[k]), h[k]);
   }
   double Q[10];
-  if (!DW) {
-    element_kernel(R, vt, at, c20, Q);
-  } else if (!face_kernel_dw(D, at, c20, 6.0 / 9.0, Q)) {
-    double e[3][3];
-    edge_vectors(coord, __ldg(tet + t), e);
-    face_kernel(compute_geo(e), at, c20, 6.0 / 9.0, Q);
-  }
+  element_kernel(R, vt, at, c20, Q);
   if (FAC) {
     double2* fo = reinterpret_cast<double2*>(factor + 10 * t);
     fo[0] = make_double2(Q[0], Q[1]);
@@ -306,7 +179,9 @@ __device__ __forceinline__ void assemble_element(int64_t t, const double* __rest
   const double base = icT * hs;
   // condensed block S[k][m] = d_k d_m (1/(c|T|) + Qf/9), each entry once, as
   // d_k (Q_km d_m + e_m) with d = sigma |F| (sign on the bit pattern) and
-  // e_m = d_m / (c|T|): 4 + 2 per entry FP64 operations
+  // e_m = d_m / (c|T|): 4 + 2 per entry FP64 operations.  (In fixed point too,
+  // from the integers behind Q: 24 FP64 operations fewer but 800 integer
+  // instructions more, 2.31 -> 2.62 ms at 17.9M tets.)
   double d[4], e4[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {

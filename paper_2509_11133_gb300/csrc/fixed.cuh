@@ -189,6 +189,49 @@ FX_HD bool geometry(const double e[3][3], int64_t g[6], int& kg, double& adet) {
 }
 
 // ---------------------------------------------------------------------------
+// |u x v|^2 of two edges of a face.  False (fp64 takes the face) when the
+// largest component of the product is below 2^-5 of the square of the largest
+// edge component -- a thin triangle, whose product would keep fewer bits than
+// fp64's -- or an exponent is out of range.
+// ---------------------------------------------------------------------------
+FX_HD bool cross_norm2(const double u[3], const double v[3], double& n2) {
+  uint32_t all = 0;
+  for (int d = 0; d < 3; ++d) {
+    const uint32_t a = (uint32_t)(bits_of(u[d]) >> 32) & 0x7FFFFFFFu, b = (uint32_t)(bits_of(v[d]) >> 32) & 0x7FFFFFFFu;
+    all = all > a ? all : a;
+    all = all > b ? all : b;
+  }
+  const int k = (int)(all >> 20) - 1023;
+  if (k < -200 || k > 200) return false;
+  Half a[3], b[3], n[3];
+  for (int d = 0; d < 3; ++d) {
+    const int64_t w = from_double(v[d], k);
+    a[d] = split(from_double(u[d], k));
+    b[d] = split(w);
+    n[d] = split(-w);
+  }
+  int64_t c[3], most = 0;
+  for (int d = 0; d < 3; ++d) {
+    const int p = (d + 1) % 3, q = (d + 2) % 3;
+    Acc s(2);
+    mac_wide(s, a[p], b[q]);
+    mac_wide(s, a[q], n[p]);
+    c[d] = shifted(s, 2);  // below 2^61: units of 2^(2k - 58)
+    const int64_t m = c[d] < 0 ? -c[d] : c[d];
+    most = most > m ? most : m;
+  }
+  if (most < ((int64_t)1 << 53)) return false;
+  const int up = clz64((uint64_t)most) - 3;  // the largest in [2^60, 2^61)
+  Acc s(2);
+  for (int d = 0; d < 3; ++d) {
+    const Half h = split((int64_t)((uint64_t)c[d] << up));
+    mac_wide(s, h, h);
+  }
+  n2 = to_double(shifted(s, 2), 4 * k - 116 - 2 * up + 62);
+  return true;
+}
+
+// ---------------------------------------------------------------------------
 // The condensation kernel Q = Qf/9 (face-indexed, packed upper triangle) of an
 // element from its fixed-point G: with M = a T0 + (c/20) G (T0 = I + 1 1'),
 //     Y = (6/9) / (|det E| det M) adj(M) G T0^-1,   G T0^-1 = G - (G 1) 1'/4,

@@ -101,76 +101,6 @@ __device__ __forceinline__ void tet_geom(const double* __restrict__ coord, int4 
   vol[t] = make_double2(adet, rdet);
 }
 
-// The double-word geometry record of tet t (meshes of ph_mesh_create_dw):
-// E, det E, |det E| and 1/|det E| in fp64 as in compute_geo (so |det E| and
-// 1/|det E| are the fp64 record's bits), then E scaled by the power of two
-// of its largest entry, G' = E'E'^T, its scale 2^kg and G'T = G' - (G' 1) 1'/4
-// in double-word (dw.cuh), stored as the layout of load_geo_dw reads it.
-__device__ __forceinline__ void tet_geom_dw(const double* __restrict__ coord, int4 v, int64_t t,
-                                            double* __restrict__ geo, double2* __restrict__ vol, unsigned* status) {
-  using namespace dw;
-  double e[3][3];
-  ph_elem::edge_vectors(coord, v, e);
-  const double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) +
-                     e[0][1] * (e[1][2] * e[2][0] - e[1][0] * e[2][2]) +
-                     e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
-  const double adet = ph::neg_if(det, __double2hiint(det) < 0);
-  if (!ph::pos_finite(adet)) ph_flag(status, PH_ERR_DEGENERATE);
-  const double rdet = ph::rcp_newton(adet);
-  int kE = -1023;
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int d = 0; d < 3; ++d) kE = max(kE, exponent(e[i][d]));
-  f2 E[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int d = 0; d < 3; ++d) E[i][d] = from_double(e[i][d], -kE);
-  f2 g[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = i; j < 3; ++j) g[i][j] = add(add(mul(E[i][0], E[j][0]), mul(E[i][1], E[j][1])), mul(E[i][2], E[j][2]));
-  const int kd = max(exponent(g[0][0].h), max(exponent(g[1][1].h), exponent(g[2][2].h)));
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = i; j < 3; ++j) g[i][j] = ldexp(g[i][j], -kd);
-  g[1][0] = g[0][1];
-  g[2][0] = g[0][2];
-  g[2][1] = g[1][2];
-  float out[36];
-  const f2 gs[6] = {g[0][0], g[0][1], g[0][2], g[1][1], g[1][2], g[2][2]};
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    out[2 * i] = gs[i].h;
-    out[2 * i + 1] = gs[i].l;
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const f2 q = ldexp(add(add(g[i][0], g[i][1]), g[i][2]), -2);  // row sum / 4 (exact scaling)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const f2 tij = sub(g[i][j], q);
-      out[12 + 2 * (3 * i + j)] = tij.h;
-      out[13 + 2 * (3 * i + j)] = tij.l;
-    }
-  }
-  const int kg = 2 * kE + kd;
-  out[30] = __int_as_float(__double2loint(adet));
-  out[31] = __int_as_float(__double2hiint(adet));
-  out[32] = __int_as_float(__double2loint(rdet));
-  out[33] = __int_as_float(__double2hiint(rdet));
-  out[34] = __int_as_float(kg);
-  out[35] = __int_as_float(-2 * exponent(rdet) - (exponent(g[0][0].h) + exponent(g[1][1].h) + exponent(g[2][2].h) +
-                                                  3 * kg));
-  vol[t] = make_double2(adet, rdet);
-  float4* o = reinterpret_cast<float4*>(geo + PH_GEO_DW_STRIDE * t);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) o[i] = make_float4(out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
-}
-
 // 1. histogram of face keys by bucket
 __global__ void k_face_count(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
                              int64_t nN, int sub, int32_t* __restrict__ cnt, int4* __restrict__ tet_copy,
@@ -202,8 +132,7 @@ constexpr int kFillThreads = 128;
 __global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
                             int64_t nN, int sub, const int32_t* __restrict__ start, int32_t* __restrict__ cnt,
                             int4* __restrict__ entries, int32_t* __restrict__ mate, const double* __restrict__ coord,
-                            double* __restrict__ geo, int32_t* __restrict__ gexp, double2* __restrict__ vol, bool geo_dw,
-                            unsigned* status) {
+                            double* __restrict__ geo, int32_t* __restrict__ gexp, double2* __restrict__ vol, unsigned* status) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (failed(status)) return;
   if (i < nE) {
@@ -221,8 +150,7 @@ __global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __res
       entries[pos[k]] = make_int4(s.x, s.y, s.z, (int)(4 * i + k));
     }
     reinterpret_cast<int4*>(mate)[i] = make_int4(-1, -1, -1, -1);  // no mate yet (boundary)
-    if (geo_dw) tet_geom_dw(coord, v, i, geo, vol, status);
-    else tet_geom(coord, v, i, geo, gexp, vol, status);
+    tet_geom(coord, v, i, geo, gexp, vol, status);
   } else if (i < nE + nN) {
     int3 f = neumann_tri(nb, i - nE);
     if (!valid_tri(f, nC)) return;
@@ -400,16 +328,21 @@ __global__ void k_face_emit(const int4* __restrict__ tet, int64_t nE, const int4
     emit_tet(t1, v1, m1, fb1, om1, ofb1, nF, tface, face_tet, face_vtx, face_kind, flag, mult_iota, tmult, rowlen);
 }
 
-// face area 1/2 |(P_z - P_x) x (P_y - P_x)|
-__device__ __forceinline__ void face_area(const double* __restrict__ coord, const int32_t* __restrict__ face_vtx,
-                                          int64_t F, double* __restrict__ area) {
-  const double* x = coord + 3 * (int64_t)face_vtx[3 * F];
-  const double* y = coord + 3 * (int64_t)face_vtx[3 * F + 1];
-  const double* z = coord + 3 * (int64_t)face_vtx[3 * F + 2];
-  double u0 = z[0] - x[0], u1 = z[1] - x[1], u2 = z[2] - x[2];
-  double v0 = y[0] - x[0], v1 = y[1] - x[1], v2 = y[2] - x[2];
-  double cx = u1 * v2 - u2 * v1, cy = u2 * v0 - u0 * v2, cz = u0 * v1 - u1 * v0;
-  area[F] = ph::half_sqrt(cx * cx + cy * cy + cz * cz);
+// face area 1/2 |(P_z - P_x) x (P_y - P_x)| of the vertices p[0..2] = P_x, P_y,
+// P_z: the product and its norm in fixed point (fixed.cuh), 12 FP64 operations
+// in place of 22
+__device__ __forceinline__ double face_area(const double p[3][3]) {
+  double u[3], v[3], n2;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    u[d] = p[2][d] - p[0][d];
+    v[d] = p[1][d] - p[0][d];
+  }
+  if (!fx::cross_norm2(u, v, n2)) {
+    const double cx = u[1] * v[2] - u[2] * v[1], cy = u[2] * v[0] - u[0] * v[2], cz = u[0] * v[1] - u[1] * v[0];
+    n2 = cx * cx + cy * cy + cz * cz;
+  }
+  return ph::half_sqrt(n2);
 }
 
 // Neumann faces get no multiplier.  Face counts are read on the device
@@ -445,6 +378,16 @@ __global__ void k_tet_mult(const int4* __restrict__ tface, int64_t nE, const int
   tmult[t] = make_int4(o[0], o[1], o[2], o[3]);
 }
 
+// last p with off[p] <= i (off ascending, off[0] = 0)
+__device__ __forceinline__ int problem_of(const int64_t* __restrict__ off, int32_t n, int64_t i) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (off[mid] <= i) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
 // The other three local faces of a tet, m != k ascending, as multiplier ids
 // (PH_NO_MULT, which sorts last, for Neumann faces or no tet).
 __device__ __forceinline__ void other_mults(int4 tm, int k, int& o0, int& o1, int& o2) {
@@ -473,38 +416,83 @@ __device__ __forceinline__ int rank7(const int c[7], int x) {
   return r;
 }
 
-// 8. column indices of each row (ascending), the diagonal position, and each
-//    slot's scatter positions: tpos = diagonal, trel = rank offsets of the
+// 8. column indices of each row (ascending) and each slot's scatter positions: tpos = diagonal, trel = rank offsets of the
 //    other three local faces (4-bit two's complement, m != k ascending).
 //    Row l(F) holds l(F) and the other non-Neumann faces of F's one or two
 //    tets (all distinct): 7 candidates with PH_NO_MULT for absent ones, put in
 //    order by a 16-comparator sorting network, all in registers.  The thread
-//    first computes the face's area (FP64), which overlaps the gathers.
-__global__ void k_row_fill(const int2* __restrict__ face_tet, const int4* __restrict__ tface,
-                           const int4* __restrict__ tmult, const int32_t* __restrict__ face_mult,
+//    also computes the face's area.  Bound by the latency of its chains of
+//    gathers (ncu: 7 of 15 cycles per issue) beside the FP64 and integer
+//    pipes, half busy each: with the area's product in fixed point and all
+//    loads issued first, 1.50 -> 1.35 ms at 35.9M faces (area alone 1.46); five
+//    blocks per SM (48 registers), 3 and 4 take 1.60 and 1.39.
+// BATCH (a batched build): U holds the problems' offsets; the face's ids (in
+// place), its column ids and positions are then local to its problem.
+struct FillOffsets {
+  const int64_t *toff, *voff;
+  const long long* first;  // first face, multiplier, CSR entry
+  int32_t n;
+};
+
+template <bool BATCH>
+__global__ void __launch_bounds__(ph::kThreads, BATCH ? 4 : 5) k_row_fill(int2* __restrict__ face_tet, const int4* __restrict__ tface,
+                           const int4* __restrict__ tmult, int32_t* __restrict__ face_mult,
                            const int64_t* __restrict__ d_tot, int64_t nFmax,
                            const int32_t* __restrict__ rowptr, int32_t* __restrict__ colind,
-                           int32_t* __restrict__ rowdiag, int32_t* __restrict__ tpos,
+                           int32_t* __restrict__ tpos,
                            unsigned short* __restrict__ trel, const double* __restrict__ coord,
-                           const int32_t* __restrict__ face_vtx, double* __restrict__ area, unsigned* status) {
+                           int32_t* __restrict__ face_vtx, double* __restrict__ area, const FillOffsets U,
+                           unsigned* status) {
   const int64_t F = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (F >= nFmax || F >= d_tot[0] || failed(status)) return;
-  face_area(coord, face_vtx, F, area);
-  const int l = face_mult[F];
-  if (l < 0) return;
+  // every load whose address is known, before anything uses one: the vertices'
+  // and the tets' chains of loads run side by side
   const int2 ft = face_tet[F];
+  const int l = face_mult[F];
   const int T[2] = {ft.x, ft.y};
+  int vtx[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) vtx[j] = face_vtx[3 * F + j];
+  int4 tf[2], tm[2];
+#pragma unroll
+  for (int side = 0; side < 2; ++side)
+    if (T[side] >= 0) {
+      tf[side] = tface[T[side]];
+      tm[side] = tmult[T[side]];
+    }
+  double p[3][3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) p[j][d] = coord[3 * (int64_t)vtx[j] + d];
+  int base = 0, end = 0;
+  if (l >= 0) {
+    base = rowptr[l];
+    end = rowptr[l + 1];
+  }
+  area[F] = face_area(p);
+  int m0 = 0, z0 = 0;
+  if (BATCH) {
+    const int q = problem_of(U.toff, U.n, T[0]);
+    const int t0 = (int)U.toff[q], v0 = (int)U.voff[q];
+    m0 = (int)U.first[3 * q + 1];
+    z0 = (int)U.first[3 * q + 2];
+    face_tet[F] = make_int2(ft.x - t0, ft.y < 0 ? -1 : ft.y - t0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) face_vtx[3 * F + j] = vtx[j] - v0;
+    if (l >= 0) face_mult[F] = l - m0;
+  }
+  if (l < 0) return;
   int k[2] = {0, 0};
   int o[2][3];
 #pragma unroll
   for (int side = 0; side < 2; ++side) {
     o[side][0] = o[side][1] = o[side][2] = PH_NO_MULT;
     if (T[side] < 0) continue;
-    const int4 tf = tface[T[side]], tm = tmult[T[side]];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      if ((comp(tf, j) & PH_ID_MASK) == F) k[side] = j;
-    other_mults(tm, k[side], o[side][0], o[side][1], o[side][2]);
+      if ((comp(tf[side], j) & PH_ID_MASK) == F) k[side] = j;
+    other_mults(tm[side], k[side], o[side][0], o[side][1], o[side][2]);
   }
   int c[7] = {l, o[0][0], o[0][1], o[0][2], o[1][0], o[1][1], o[1][2]};
   cswap(c[0], c[6]); cswap(c[2], c[3]); cswap(c[4], c[5]);
@@ -515,13 +503,11 @@ __global__ void k_row_fill(const int2* __restrict__ face_tet, const int4* __rest
   cswap(c[1], c[2]); cswap(c[3], c[4]); cswap(c[5], c[6]);
   const int n = 7 - ((c[0] == PH_NO_MULT) + (c[1] == PH_NO_MULT) + (c[2] == PH_NO_MULT) + (c[3] == PH_NO_MULT) +
                      (c[4] == PH_NO_MULT) + (c[5] == PH_NO_MULT) + (c[6] == PH_NO_MULT));
-  const int base = rowptr[l];
-  if (rowptr[l + 1] - base != n) { ph_flag(status, PH_ERR_ARG); return; }
+  if (end - base != n) { ph_flag(status, PH_ERR_ARG); return; }
 #pragma unroll
   for (int i = 0; i < 7; ++i)
-    if (i < n) colind[base + i] = c[i];
-  const int rl = rank7(c, l);
-  rowdiag[l] = base + rl;
+    if (i < n) colind[base + i] = c[i] - m0;
+  const int rl = rank7(c, l), diag = base + rl - z0;
 #pragma unroll
   for (int side = 0; side < 2; ++side) {
     if (T[side] < 0) continue;
@@ -531,7 +517,7 @@ __global__ void k_row_fill(const int2* __restrict__ face_tet, const int4* __rest
       const int lm = o[side][idx];
       if (lm != PH_NO_MULT) bits |= ((unsigned)(rank7(c, lm) - rl) & 0xFu) << (4 * idx);
     }
-    tpos[4 * (int64_t)T[side] + k[side]] = base + rl;
+    tpos[4 * (int64_t)T[side] + k[side]] = diag;
     trel[4 * (int64_t)T[side] + k[side]] = (unsigned short)bits;
   }
 }
@@ -603,7 +589,7 @@ __global__ void k_batch_offsets(const int4* __restrict__ tface, const int32_t* _
 // Hook of a batched build: the per-problem offsets, computed before the
 // build's one synchronisation and read with it.
 struct BatchCounts {
-  const int64_t* d_toff;  // n + 1 tet offsets (device)
+  const int64_t *d_toff, *d_voff;  // n + 1 tet and vertex offsets (device)
   int32_t n;
   long long* d_counts;  // 3n: first face, multiplier, CSR entry of each problem
   long long* h_counts;  // 3n (host)
@@ -665,13 +651,13 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   // first part zeroed by one memset).  Few host calls keep the GPU fed.
   Carve mc, sc;
   const size_t o_status = mc.take<unsigned>(1), o_coord = mc.take<double>(3 * nC), o_tet = mc.take<int4>(nE);
-  const size_t o_geo = mc.take<double>((dw ? PH_GEO_DW_STRIDE : PH_GEO_STRIDE) * nE), o_tface = mc.take<int4>(nE);
-  const size_t o_gexp = mc.take<int32_t>(dw ? 0 : nE), o_vol = mc.take<double2>(nE);
+  const size_t o_geo = mc.take<double>(PH_GEO_STRIDE * nE), o_tface = mc.take<int4>(nE);
+  const size_t o_gexp = mc.take<int32_t>(nE), o_vol = mc.take<double2>(nE);
   const size_t o_tmult = mc.take<int4>(nE), o_tpos = mc.take<int4>(nE), o_trel = mc.take<ushort4>(nE);
   const size_t o_ftet = mc.take<int2>(nFmax), o_fvtx = mc.take<int32_t>(3 * nFmax);
   const size_t o_fkind = mc.take<int8_t>(nFmax), o_fmult = mc.take<int32_t>(nFmax + 1);
   const size_t o_farea = mc.take<double>(nFmax), o_rowptr = mc.take<int32_t>(nFmax + 1);
-  const size_t o_colind = mc.take<int32_t>(nnzmax), o_rowdiag = mc.take<int32_t>(nFmax);
+  const size_t o_colind = mc.take<int32_t>(nnzmax);
   // scratch: zeroed part first
   const size_t o_tot = sc.take<int64_t>(3), o_cnt = sc.take<int32_t>(nb);
   const size_t o_s1 = sc.take<unsigned long long>(scan_state_words(nb));
@@ -709,7 +695,6 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
     m->face_area = Carve::at<double>(A, o_farea);
     m->rowptr = Carve::at<int32_t>(A, o_rowptr);
     m->colind = Carve::at<int32_t>(A, o_colind);
-    m->rowdiag = Carve::at<int32_t>(A, o_rowdiag);
   }
   {
   int64_t* d_tot = Carve::at<int64_t>(scratch, o_tot);  // [0] nF, [1] L, [2] nnz
@@ -740,7 +725,7 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
     {
       KernelTimer kt("k_face_fill", s, 2);
       k_face_fill<<<grid_for(nE + nN, kFillThreads), kFillThreads, 0, s>>>(m->tet, nE, nC, neumann, nN, sub, start, cnt, entries,
-                                                         mate, m->coord, m->geo, m->gexp, m->vol, dw, m->status);
+                                                         mate, m->coord, m->geo, m->gexp, m->vol, m->status);
       PH_CU(launched(), "k_face_fill");
     }
     {
@@ -775,22 +760,27 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   }
   PH_TRY(exclusive_scan(rowlen, m->rowptr, nFmax + 1, d_tot + 2, s, m->status, d_tot + 1, 1, st4));  // nnz
 
-  // --- CSR columns and scatter positions (slots without a multiplier are never read)
-  if (nFmax > 0) {
-    KernelTimer kt("k_row_fill", s, 2);
-    k_row_fill<<<gF, kThreads, 0, s>>>(m->face_tet, m->tface, m->tmult, m->face_mult, d_tot, nFmax, m->rowptr,
-                                       m->colind, m->rowdiag, reinterpret_cast<int32_t*>(m->tpos),
-                                       reinterpret_cast<unsigned short*>(m->trel), m->coord, m->face_vtx,
-                                       m->face_area, m->status);
-    PH_CU(launched(), "k_row_fill");
-  }
   if (bc && bc->n > 0) {  // per-problem offsets of a batched build
     k_batch_offsets<<<grid_for(bc->n), kThreads, 0, s>>>(m->tface, m->face_mult, m->rowptr, d_tot, bc->d_toff, bc->n,
                                                          bc->d_counts, m->status);
     PH_CU(launched(), "k_batch_offsets");
+  }
+
+  // --- CSR columns and scatter positions (slots without a multiplier are never read)
+  if (nFmax > 0) {
+    KernelTimer kt("k_row_fill", s, 2);
+    const auto fill = bc ? k_row_fill<true> : k_row_fill<false>;
+    fill<<<gF, kThreads, 0, s>>>(m->face_tet, m->tface, m->tmult, m->face_mult, d_tot, nFmax, m->rowptr, m->colind,
+                                 reinterpret_cast<int32_t*>(m->tpos), reinterpret_cast<unsigned short*>(m->trel),
+                                 m->coord, m->face_vtx, m->face_area,
+                                 bc ? FillOffsets{bc->d_toff, bc->d_voff, bc->d_counts, bc->n}
+                                    : FillOffsets{nullptr, nullptr, nullptr, 0},
+                                 m->status);
+    PH_CU(launched(), "k_row_fill");
+  }
+  if (bc && bc->n > 0)
     PH_CU(cudaMemcpyAsync(bc->h_counts, bc->d_counts, sizeof(long long) * 3 * bc->n, cudaMemcpyDeviceToHost, s),
           "copy");
-  }
   // the one synchronisation: counts and the first error of any kernel
   PH_TRY(read_counters(d_tot, 3, m->status, s, tot, &bits));
   }
@@ -898,16 +888,6 @@ struct UnionOffsets {
   int32_t n;
 };
 
-// last p with off[p] <= i (off ascending, off[0] = 0)
-__device__ __forceinline__ int problem_of(const int64_t* __restrict__ off, int32_t n, int64_t i) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= i) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 struct UnionSources {
   const int32_t* tet;  // problem's tets (nE_p x 4)
   const int32_t* nb;   // problem's Neumann triples or null
@@ -943,13 +923,15 @@ __device__ __forceinline__ int shift_id(int x, int64_t off) {  // keep bit 31 (s
   return (int)(((unsigned)x & 0x80000000u) | (unsigned)((x & PH_ID_MASK) - (int)off));
 }
 
-// per tet: local vertex ids, face ids, multiplier ids, CSR positions
+// per tet: local vertex ids, face ids, multiplier ids (k_row_fill has made the
+// faces' and the CSR's local: separate passes over the 521M columns and 75M
+// faces of 256 problems took 2.3 and 0.7 ms)
 __global__ void k_rebase_tets(UnionOffsets o, int64_t nE, int4* __restrict__ tet, int4* __restrict__ tface,
-                              int4* __restrict__ tmult, int4* __restrict__ tpos) {
+                              int4* __restrict__ tmult) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
   const int p = problem_of(o.toff, o.n, t);
-  const int v = (int)o.voff[p], z = (int)o.zoff[p];
+  const int v = (int)o.voff[p];
   const int64_t f = o.foff[p], mo = o.moff[p];
   const int4 a = tet[t];
   tet[t] = make_int4(a.x - v, a.y - v, a.z - v, a.w - v);
@@ -961,48 +943,22 @@ __global__ void k_rebase_tets(UnionOffsets o, int64_t nE, int4* __restrict__ tet
   for (int k = 0; k < 4; ++k)
     if (cm[k] != PH_NO_MULT) cm[k] = shift_id(cm[k], mo);
   tmult[t] = make_int4(cm[0], cm[1], cm[2], cm[3]);
-  const int4 d = tpos[t];  // positions of Neumann slots are never read
-  tpos[t] = make_int4(d.x - z, d.y - z, d.z - z, d.w - z);
-}
-
-// per face: local T+/T-, vertex ids and multiplier id
-__global__ void k_rebase_faces(UnionOffsets o, int64_t nF, int2* __restrict__ face_tet,
-                               int32_t* __restrict__ face_vtx, int32_t* __restrict__ face_mult) {
-  const int64_t F = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (F >= nF) return;
-  const int p = problem_of(o.foff, o.n, F);
-  const int t0 = (int)o.toff[p], v = (int)o.voff[p];
-  const int2 ft = face_tet[F];
-  face_tet[F] = make_int2(ft.x - t0, ft.y < 0 ? -1 : ft.y - t0);
-  face_vtx[3 * F] -= v;
-  face_vtx[3 * F + 1] -= v;
-  face_vtx[3 * F + 2] -= v;
-  const int l = face_mult[F];
-  if (l >= 0) face_mult[F] = l - (int)o.moff[p];
 }
 
 // per multiplier row: the problem's own row pointers (problem p's L_p + 1
-// entries at rowptr_b + moff[p] + p) and diagonal positions
+// entries at rowptr_b + moff[p] + p)
 __global__ void k_rebase_rows(UnionOffsets o, int64_t L, const int32_t* __restrict__ rowptr,
-                              int32_t* __restrict__ rowptr_b, int32_t* __restrict__ rowdiag) {
+                              int32_t* __restrict__ rowptr_b) {
   const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (l >= L + o.n) return;
   if (l < L) {
     const int p = problem_of(o.moff, o.n, l);
     const int z = (int)o.zoff[p];
     rowptr_b[l + p] = rowptr[l] - z;
-    rowdiag[l] -= z;
   } else {  // the closing entry of problem p: its nnz
     const int p = (int)(l - L);
     rowptr_b[o.moff[p + 1] + p] = (int)(o.zoff[p + 1] - o.zoff[p]);
   }
-}
-
-// per CSR entry: local column ids
-__global__ void k_rebase_cols(UnionOffsets o, int64_t nnz, int32_t* __restrict__ colind) {
-  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (j >= nnz) return;
-  colind[j] -= (int)o.moff[problem_of(o.zoff, o.n, j)];
 }
 
 }  // namespace
@@ -1065,7 +1021,7 @@ extern "C" ph_status ph_mesh_create_batch(int32_t n, const double* const* coord,
     return cuda_status(e, "ph_mesh_create_batch inputs");
   }
   std::vector<long long> cnt(3 * (size_t)n, -1);
-  BatchCounts bc{d_off, n, d_cnt, cnt.data()};
+  BatchCounts bc{d_off, d_off + 2 * (n + 1), n, d_cnt, cnt.data()};
   ph_mesh* u = nullptr;
   ph_status st = mesh_build(coord_u, nCu, reinterpret_cast<const int32_t*>(tet_u), nEu, nNu > 0 ? nb_u : nullptr,
                             nNu, s, &u, &bc);
@@ -1105,19 +1061,11 @@ extern "C" ph_status ph_mesh_create_batch(int32_t n, const double* const* coord,
   e = cudaMemcpyAsync(tab, t5.data(), sizeof(int64_t) * t5.size(), cudaMemcpyHostToDevice, s);
   const UnionOffsets o{tab, tab + (n + 1), tab + 2 * (n + 1), tab + 3 * (n + 1), tab + 4 * (n + 1), n};
   if (e == cudaSuccess && nEu > 0) {
-    k_rebase_tets<<<grid_for(nEu), kThreads, 0, s>>>(o, nEu, u->tet, u->tface, u->tmult, u->tpos);
-    e = launched();
-  }
-  if (e == cudaSuccess && u->nF > 0) {
-    k_rebase_faces<<<grid_for(u->nF), kThreads, 0, s>>>(o, u->nF, u->face_tet, u->face_vtx, u->face_mult);
+    k_rebase_tets<<<grid_for(nEu), kThreads, 0, s>>>(o, nEu, u->tet, u->tface, u->tmult);
     e = launched();
   }
   if (e == cudaSuccess) {
-    k_rebase_rows<<<grid_for(u->L + n), kThreads, 0, s>>>(o, u->L, u->rowptr, rowptr_b, u->rowdiag);
-    e = launched();
-  }
-  if (e == cudaSuccess && u->nnz > 0) {
-    k_rebase_cols<<<grid_for(u->nnz), kThreads, 0, s>>>(o, u->nnz, u->colind);
+    k_rebase_rows<<<grid_for(u->L + n), kThreads, 0, s>>>(o, u->L, u->rowptr, rowptr_b);
     e = launched();
   }
   if (e != cudaSuccess) {
@@ -1160,7 +1108,6 @@ extern "C" ph_status ph_mesh_create_batch(int32_t n, const double* const* coord,
     m->face_area = u->face_area + f0;
     m->rowptr = rowptr_b + m0 + p;
     m->colind = u->colind + z0;
-    m->rowdiag = u->rowdiag + m0;
     m->status = u->status;
     out[p] = m;
   }

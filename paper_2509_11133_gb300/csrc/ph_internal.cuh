@@ -16,10 +16,9 @@
 #define PH_ID_MASK 0x7FFFFFFF
 // Per-element geometry record: G_e = E E' (00 01 02 11 12 22) as six int64 on
 // the element's scale 2^gexp (fixed.cuh), or as six doubles where gexp is
-// PH_GEXP_F64.  Meshes of ph_mesh_create_dw: 18 doubles (element.cuh).
+// PH_GEXP_F64.
 #define PH_GEO_STRIDE 6
 #define PH_GEXP_F64 INT32_MIN
-#define PH_GEO_DW_STRIDE 18
 
 // Device memory shared by the meshes of one batched build (ph_mesh_create_batch):
 // released when the last of them is destroyed.
@@ -40,8 +39,8 @@ struct ph_mesh {
   int4* tmult;         // nE: see PH_NO_MULT / PH_BND_BIT
   int4* tpos;          // nE: CSR position of the diagonal entry of row l(F_k)
   ushort4* trel;       // nE: 3 packed 4-bit offsets (m != k, ascending m) from tpos
-  double* geo;         // nE*PH_GEO_STRIDE (PH_GEO_DW_STRIDE): the geometry record
-  int32_t* gexp;       // nE: scale of the record (not in a double-word mesh)
+  double* geo;         // nE*PH_GEO_STRIDE: the geometry record
+  int32_t* gexp;       // nE: scale of the record
   double2* vol;        // nE: |det E|, 1/|det E|
   int2* face_tet;      // nF
   int32_t* face_vtx;   // nF*3
@@ -50,9 +49,8 @@ struct ph_mesh {
   double* face_area;   // nF
   int32_t* rowptr;     // L+1
   int32_t* colind;     // nnz
-  int32_t* rowdiag;    // L
   unsigned int* status;  // device status word: bit s set for ph_status s
-  bool geo_dw;           // geo holds the double-word record (ph_mesh_create_dw)
+  bool geo_dw;           // from ph_mesh_create_dw: refused by the fp64 entry points
 };
 
 namespace ph {

@@ -28,6 +28,7 @@ extern "C" int run(const double* e, double a, double c20, double* adet, double* 
   if (!fx::geometry(E, g, kg, *adet)) return 0;
   return fx::face_kernel(g, kg, a, c20, 1.0 / *adet, [](double x) { return 1.0 / x; }, Q) ? 2 : 1;
 }
+extern "C" int norm2(const double* u, const double* v, double* n2) { return fx::cross_norm2(u, v, *n2); }
 extern "C" double there_and_back(double x, int k) { return fx::to_double(fx::from_double(x, k), k - 60); }
 """
 
@@ -43,6 +44,7 @@ def lib(tmp_path_factory):
     L = ctypes.CDLL(str(so))
     D = ctypes.c_double
     L.run.argtypes = [ctypes.POINTER(D), D, D, ctypes.POINTER(D), ctypes.POINTER(D)]
+    L.norm2.argtypes = [ctypes.POINTER(D), ctypes.POINTER(D), ctypes.POINTER(D)]
     L.there_and_back.argtypes, L.there_and_back.restype = [D, ctypes.c_int], D
     return L
 
@@ -115,6 +117,26 @@ def test_against_rationals(lib, kind):
             big = max(abs(x) for x in ref)
             assert max(abs(Fraction(float(q)) - x) for q, x in zip(Q, ref)) <= Fraction(tol + 8 * 2.0 ** -53) * big
     assert taken >= 60
+
+
+@pytest.mark.parametrize("thin", [1.0, 0.1, 0.02, 1e-4])
+def test_cross_norm(lib, thin):
+    """|u x v|^2: the components round at 2 units of 2^-60 of the square of the
+    largest edge component, and the largest of them is at least 2^-7 of it."""
+    P = ctypes.POINTER(ctypes.c_double)
+    rng = np.random.default_rng(4)
+    taken = 0
+    for _ in range(300):
+        u = rng.standard_normal(3) * 10.0 ** rng.uniform(-6, 6)
+        v = 0.7 * u + thin * np.abs(u).max() * rng.standard_normal(3)
+        n2 = ctypes.c_double()
+        if not lib.norm2(u.ctypes.data_as(P), v.ctypes.data_as(P), ctypes.byref(n2)):
+            continue
+        taken += 1
+        a, b = [Fraction(float(x)) for x in u], [Fraction(float(x)) for x in v]
+        ref = sum((a[i - 2] * b[i - 1] - a[i - 1] * b[i - 2]) ** 2 for i in range(3))
+        assert abs(Fraction(n2.value) - ref) <= Fraction(2.0 ** -53 + 8 * 2.0 ** -53) * ref
+    assert taken >= 200 if thin >= 0.1 else taken < 300 if thin > 1e-3 else taken == 0
 
 
 def test_left_to_fp64(lib):
