@@ -41,14 +41,15 @@ __device__ __forceinline__ void faces_of_edge(int j, int& a, int& b) {
 // and the edge's vertex pair (written by its first occurrence).
 __global__ void k_patch_count(const int4* __restrict__ tet, const int4* __restrict__ tface,
                               const int4* __restrict__ tmult, int64_t nE, const int32_t* __restrict__ first,
-                              const int32_t* __restrict__ ebase, int32_t* __restrict__ cnt, int2* __restrict__ ev) {
+                              const int32_t* __restrict__ ebase, const uint8_t* __restrict__ mask,
+                              int32_t* __restrict__ cnt, int2* __restrict__ ev) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
   const int4 v = tet[t], tf = tface[t], tm = tmult[t];
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
     const int64_t slot = 6 * t + j;
-    const int e = edge_id(first, ebase, slot);
+    const int e = edge_id(first, ebase, mask, slot);
     if (first[slot] == (int)slot) {
       int p, q;
       local_edge(j, p, q);
@@ -64,13 +65,14 @@ __global__ void k_patch_count(const int4* __restrict__ tet, const int4* __restri
 
 __global__ void k_patch_fill(const int4* __restrict__ tface, const int4* __restrict__ tmult, int64_t nE,
                              const int32_t* __restrict__ first, const int32_t* __restrict__ ebase,
-                             const int32_t* __restrict__ off, int32_t* __restrict__ fill, int32_t* __restrict__ mem) {
+                             const uint8_t* __restrict__ mask, const int32_t* __restrict__ off,
+                             int32_t* __restrict__ fill, int32_t* __restrict__ mem) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
   const int4 tf = tface[t], tm = tmult[t];
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
-    const int e = edge_id(first, ebase, 6 * t + j);
+    const int e = edge_id(first, ebase, mask, 6 * t + j);
     int f2[2];
     faces_of_edge(j, f2[0], f2[1]);
 #pragma unroll
@@ -302,7 +304,7 @@ extern "C" ph_status ph_schwarz_create(const ph_mesh* m, const double* values, v
   if (e == cudaSuccess) e = cudaMemsetAsync(fill, 0, sizeof(int32_t) * (P->nEd + 1), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(gcnt, 0, sizeof(int32_t) * (kSchwarzDense + 1), s);
   if (e == cudaSuccess && nE > 0) {
-    k_patch_count<<<grid_for(nE), kThreads, 0, s>>>(m->tet, m->tface, m->tmult, nE, E.first, E.ebase, cnt, ev);
+    k_patch_count<<<grid_for(nE), kThreads, 0, s>>>(m->tet, m->tface, m->tmult, nE, E.first, E.ebase, E.mask, cnt, ev);
     e = launched();
   }
   if (e != cudaSuccess) { st = cuda_status(e, "ph_schwarz_create"); goto done; }
@@ -314,7 +316,7 @@ extern "C" ph_status ph_schwarz_create(const ph_mesh* m, const double* values, v
   P->nmem = tot[1];
   e = alloc(&emem, (size_t)P->nmem, s);
   if (e == cudaSuccess && nE > 0) {
-    k_patch_fill<<<grid_for(nE), kThreads, 0, s>>>(m->tface, m->tmult, nE, E.first, E.ebase, off, fill, emem);
+    k_patch_fill<<<grid_for(nE), kThreads, 0, s>>>(m->tface, m->tmult, nE, E.first, E.ebase, E.mask, off, fill, emem);
     e = launched();
   }
   if (e == cudaSuccess && P->nEd > 0) {
