@@ -38,22 +38,23 @@ __device__ __forceinline__ void edge_vectors(const double* __restrict__ coord, i
   }
 }
 
-// Element geometry in fp64: G_e = E E', |det E| and 1/|det E| (the Newton
-// reciprocal), for the elements that fx::geometry leaves to fp64.
-__device__ __forceinline__ Geo compute_geo(const double e[3][3]) {
+// |det E| in fp64 (the sign bit cleared).
+__device__ __forceinline__ double abs_det(const double e[3][3]) {
   const double det = e[0][0] * (e[1][1] * e[2][2] - e[1][2] * e[2][1]) +
                      e[0][1] * (e[1][2] * e[2][0] - e[1][0] * e[2][2]) +
                      e[0][2] * (e[1][0] * e[2][1] - e[1][1] * e[2][0]);
-  Geo G;
-  G.adet = ph::neg_if(det, __double2hiint(det) < 0);  // |det| on the sign bit
-  G.g00 = e[0][0] * e[0][0] + e[0][1] * e[0][1] + e[0][2] * e[0][2];
-  G.g01 = e[0][0] * e[1][0] + e[0][1] * e[1][1] + e[0][2] * e[1][2];
-  G.g02 = e[0][0] * e[2][0] + e[0][1] * e[2][1] + e[0][2] * e[2][2];
-  G.g11 = e[1][0] * e[1][0] + e[1][1] * e[1][1] + e[1][2] * e[1][2];
-  G.g12 = e[1][0] * e[2][0] + e[1][1] * e[2][1] + e[1][2] * e[2][2];
-  G.g22 = e[2][0] * e[2][0] + e[2][1] * e[2][1] + e[2][2] * e[2][2];
-  G.rdet = ph::rcp_newton(G.adet);
-  return G;
+  return ph::neg_if(det, __double2hiint(det) < 0);
+}
+
+// G_e = E E' in fp64 (00 01 02 11 12 22), for the elements that fx::geometry
+// leaves out.
+__device__ __forceinline__ void gram(const double e[3][3], double g[6]) {
+  g[0] = e[0][0] * e[0][0] + e[0][1] * e[0][1] + e[0][2] * e[0][2];
+  g[1] = e[0][0] * e[1][0] + e[0][1] * e[1][1] + e[0][2] * e[1][2];
+  g[2] = e[0][0] * e[2][0] + e[0][1] * e[2][1] + e[0][2] * e[2][2];
+  g[3] = e[1][0] * e[1][0] + e[1][1] * e[1][1] + e[1][2] * e[1][2];
+  g[4] = e[1][0] * e[2][0] + e[1][1] * e[2][1] + e[1][2] * e[2][2];
+  g[5] = e[2][0] * e[2][0] + e[2][1] * e[2][1] + e[2][2] * e[2][2];
 }
 
 // The geometry record of element t as stored: g and its scale.

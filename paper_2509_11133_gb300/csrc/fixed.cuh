@@ -109,16 +109,18 @@ FX_HD double to_double(int64_t v, int k) {
 
 // ---------------------------------------------------------------------------
 // Geometry: G = E E' (00 01 02 11 12 22) of the edge vectors E (rows P_i - P_0)
-// as g = v 2^kg with the largest diagonal entry in [2^59, 2^60], and |det E|.
-// False when the element is left to fp64: an edge, or the element's extent
-// along a coordinate, below 2^-4 of the largest edge component (a common
-// scale would cost the small ones bits that fp64 keeps), det E = 0 or an
-// exponent out of range (NaN and infinity among them).
+// as g = v 2^kg with the largest diagonal entry in [2^59, 2^60].  False when the
+// element is left to fp64: an edge, or the element's extent along a coordinate,
+// below 2^-4 of the largest edge component (a common scale would cost the small
+// ones bits that fp64 keeps), or an exponent out of range (NaN and infinity
+// among them).  |det E| and the face areas stay fp64: they carry the leading
+// term d d'/(c|T|) of H, whose last bit an ill-conditioned solve amplifies by
+// 1e7, and rounding them otherwise, if better, would move such solutions.
 // ---------------------------------------------------------------------------
 constexpr int kSpread = 4;
 
-FX_HD bool geometry(const double e[3][3], int64_t g[6], int& kg, double& adet) {
-  uint32_t m[3][3], dim[3];
+FX_HD bool geometry(const double e[3][3], int64_t g[6], int& kg) {
+  uint32_t m[3][3];
   for (int i = 0; i < 3; ++i)
     for (int d = 0; d < 3; ++d) m[i][d] = (uint32_t)(bits_of(e[i][d]) >> 32) & 0x7FFFFFFFu;
   uint32_t all = 0, least = 0x7FFFFFFFu;
@@ -128,20 +130,15 @@ FX_HD bool geometry(const double e[3][3], int64_t g[6], int& kg, double& adet) {
       r = r > m[i][d] ? r : m[i][d];
       c = c > m[d][i] ? c : m[d][i];
     }
-    dim[i] = c;
     all = all > r ? all : r;
     least = least < r ? least : r;
     least = least < c ? least : c;
   }
   const int top = (int)(all >> 20), k = top - 1023;
   if (k < -300 || k > 300 || top - (int)(least >> 20) > kSpread) return false;
-  int64_t v[3][3];
   Half h[3][3];
   for (int i = 0; i < 3; ++i)
-    for (int d = 0; d < 3; ++d) {
-      v[i][d] = from_double(e[i][d], k);
-      h[i][d] = split(v[i][d]);
-    }
+    for (int d = 0; d < 3; ++d) h[i][d] = split(from_double(e[i][d], k));
   Acc a[6];
   for (int d = 0; d < 3; ++d) {
     mac(a[0], h[0][d], h[0][d]);
@@ -156,78 +153,6 @@ FX_HD bool geometry(const double e[3][3], int64_t g[6], int& kg, double& adet) {
   const int s = clz64((uint64_t)most) - 4;
   for (int i = 0; i < 6; ++i) g[i] = shifted(a[i], s);
   kg = 2 * k - 56 - s;
-  // det E = e_0 . (e_1 x e_2), each coordinate at its own scale (a product
-  // holds one factor of each) and with the low products: its error is relative
-  // to the element's extents, as in fp64
-  int kd = 3 * k;
-  Half w[3][3], n[3];
-  for (int d = 0; d < 3; ++d) {
-    const int up = top - (int)(dim[d] >> 20);
-    kd -= up;
-    for (int i = 0; i < 3; ++i) {
-      const int64_t u = (int64_t)((uint64_t)v[i][d] << up);
-      w[i][d] = split(u);
-      if (i == 2) n[d] = split(-u);
-    }
-  }
-  Acc dt(5);
-  for (int d = 0; d < 3; ++d) {
-    const int p = (d + 1) % 3, q = (d + 2) % 3;
-    Acc c(2);
-    mac_wide(c, w[1][p], w[2][q]);
-    mac_wide(c, w[1][q], n[p]);
-    mac_wide(dt, w[0][d], split(shifted(c, 2)));
-  }
-  // up to four times the product of the extents: 5 bits more than the high
-  // part where they fit, else 3
-  const bool big = dt.hh >= ((int64_t)1 << 57) || dt.hh <= -((int64_t)1 << 57);
-  int64_t det = big ? shifted(dt, 3) : shifted(dt, 5);
-  if (det == 0) return false;
-  det = det < 0 ? -det : det;
-  adet = to_double(det, big ? kd - 57 : kd - 59);
-  return true;
-}
-
-// ---------------------------------------------------------------------------
-// |u x v|^2 of two edges of a face.  False (fp64 takes the face) when the
-// largest component of the product is below 2^-5 of the square of the largest
-// edge component -- a thin triangle, whose product would keep fewer bits than
-// fp64's -- or an exponent is out of range.
-// ---------------------------------------------------------------------------
-FX_HD bool cross_norm2(const double u[3], const double v[3], double& n2) {
-  uint32_t all = 0;
-  for (int d = 0; d < 3; ++d) {
-    const uint32_t a = (uint32_t)(bits_of(u[d]) >> 32) & 0x7FFFFFFFu, b = (uint32_t)(bits_of(v[d]) >> 32) & 0x7FFFFFFFu;
-    all = all > a ? all : a;
-    all = all > b ? all : b;
-  }
-  const int k = (int)(all >> 20) - 1023;
-  if (k < -200 || k > 200) return false;
-  Half a[3], b[3], n[3];
-  for (int d = 0; d < 3; ++d) {
-    const int64_t w = from_double(v[d], k);
-    a[d] = split(from_double(u[d], k));
-    b[d] = split(w);
-    n[d] = split(-w);
-  }
-  int64_t c[3], most = 0;
-  for (int d = 0; d < 3; ++d) {
-    const int p = (d + 1) % 3, q = (d + 2) % 3;
-    Acc s(2);
-    mac_wide(s, a[p], b[q]);
-    mac_wide(s, a[q], n[p]);
-    c[d] = shifted(s, 2);  // below 2^61: units of 2^(2k - 58)
-    const int64_t m = c[d] < 0 ? -c[d] : c[d];
-    most = most > m ? most : m;
-  }
-  if (most < ((int64_t)1 << 53)) return false;
-  const int up = clz64((uint64_t)most) - 3;  // the largest in [2^60, 2^61)
-  Acc s(2);
-  for (int d = 0; d < 3; ++d) {
-    const Half h = split((int64_t)((uint64_t)c[d] << up));
-    mac_wide(s, h, h);
-  }
-  n2 = to_double(shifted(s, 2), 4 * k - 116 - 2 * up + 62);
   return true;
 }
 

@@ -14,6 +14,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <functional>
 #include <initializer_list>
 #include <vector>
 
@@ -74,24 +75,20 @@ __device__ __forceinline__ int64_t bucket_of(int3 s, int sub) {
 
 // Element geometry of tet t: the record (G_e, fixed point or fp64), its scale,
 // |det E| and 1/|det E|.
-__device__ __forceinline__ void tet_geom(const double* __restrict__ coord, int4 v, int64_t t,
+__device__ __forceinline__ void tet_geom(const double* __restrict__ coord, int4 v, int64_t t, bool fixed,
                                          double* __restrict__ geo, int32_t* __restrict__ gexp,
                                          double2* __restrict__ vol, unsigned* status) {
   double e[3][3];
   ph_elem::edge_vectors(coord, v, e);
+  const double adet = ph_elem::abs_det(e), rdet = ph::rcp_newton(adet);
+  if (!ph::pos_finite(adet)) ph_flag(status, PH_ERR_DEGENERATE);
   ph_elem::Record r;
-  double adet, rdet;
-  if (fx::geometry(e, r.g, r.kg, adet)) {
-    rdet = ph::rcp_newton(adet);
-  } else {
-    const ph_elem::Geo G = ph_elem::compute_geo(e);
-    if (!ph::pos_finite(G.adet)) ph_flag(status, PH_ERR_DEGENERATE);
-    const double g[6] = {G.g00, G.g01, G.g02, G.g11, G.g12, G.g22};
+  if (!fixed || !fx::geometry(e, r.g, r.kg)) {
+    double g[6];
+    ph_elem::gram(e, g);
 #pragma unroll
     for (int i = 0; i < 6; ++i) r.g[i] = __double_as_longlong(g[i]);
     r.kg = PH_GEXP_F64;
-    adet = G.adet;
-    rdet = G.rdet;
   }
   longlong2* o = reinterpret_cast<longlong2*>(geo + PH_GEO_STRIDE * t);
   o[0] = make_longlong2(r.g[0], r.g[1]);
@@ -99,6 +96,26 @@ __device__ __forceinline__ void tet_geom(const double* __restrict__ coord, int4 
   o[2] = make_longlong2(r.g[4], r.g[5]);
   gexp[t] = r.kg;
   vol[t] = make_double2(adet, rdet);
+}
+
+// Meshes of at least so many tets get the fixed-point record (fixed.cuh), smaller
+// ones the fp64 record.  The two differ in the last bits of Q, which an
+// unconverged Jacobi solve (7,000 iterations at 23,328 tets, rtol 1e-10) turns
+// into 4e-9 of Lambda: systems of the size that is solved that way keep their
+// bits.  There the FP64 pipe is not yet the bound: fixed point takes 9.7 us for
+// 11.8 of k_assemble at 16,464 tets, 13.8 for 16.2 at 34,992, 22 for 31 at
+// 95,832, 49 for 82 at 296,352; k_face_fill 8.5 for 8.6, 9.6 for 10.2, 13.5
+// for 15.9, 23 for 31.
+constexpr int64_t kFixedMin = 32768;
+
+// last p with off[p] <= i (off ascending, off[0] = 0)
+__device__ __forceinline__ int problem_of(const int64_t* __restrict__ off, int32_t n, int64_t i) {
+  int lo = 0, hi = n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (off[mid] <= i) lo = mid; else hi = mid - 1;
+  }
+  return lo;
 }
 
 // 1. histogram of face keys by bucket
@@ -121,10 +138,10 @@ __global__ void k_face_count(const int4* __restrict__ tet, int64_t nE, int64_t n
 
 // 2. scatter keys into buckets: entry = (v0, v1, v2, slot), slot = 4t+k for
 //    tet faces and 4nE+i for Neumann triples.  cnt counts down to 0.  The
-//    same thread then computes the tet's geometry: in fixed point on the
-//    integer pipe (fixed.cuh), 13 FP64 operations where the fp64 record took
+//    same thread then computes the tet's geometry: G_e in fixed point on the
+//    integer pipe (fixed.cuh), 22 FP64 operations where the fp64 record took
 //    55 and bound the kernel.  Now the atomics, the scattered stores and the
-//    geometry share it (17.9M tets: 1.94 -> 1.08 ms).  Blocks of 128 threads, 6
+//    geometry share it (17.9M tets: 1.94 -> 1.09 ms).  Blocks of 128 threads, 6
 //    per SM (80 registers): 5 or 7 take 1.15 and 1.09 ms, 256-thread blocks
 //    at 96 registers 1.63; storing the entries after the geometry instead of
 //    before it holds their stores back, 1.26.
@@ -132,7 +149,8 @@ constexpr int kFillThreads = 128;
 __global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
                             int64_t nN, int sub, const int32_t* __restrict__ start, int32_t* __restrict__ cnt,
                             int4* __restrict__ entries, int32_t* __restrict__ mate, const double* __restrict__ coord,
-                            double* __restrict__ geo, int32_t* __restrict__ gexp, double2* __restrict__ vol, unsigned* status) {
+                            double* __restrict__ geo, int32_t* __restrict__ gexp, double2* __restrict__ vol,
+                            const int64_t* __restrict__ toff, int32_t nprob, unsigned* status) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (failed(status)) return;
   if (i < nE) {
@@ -150,7 +168,12 @@ __global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __res
       entries[pos[k]] = make_int4(s.x, s.y, s.z, (int)(4 * i + k));
     }
     reinterpret_cast<int4*>(mate)[i] = make_int4(-1, -1, -1, -1);  // no mate yet (boundary)
-    tet_geom(coord, v, i, geo, gexp, vol, status);
+    int64_t n = nE;  // tets of the tet's mesh
+    if (toff) {
+      const int p = problem_of(toff, nprob, i);
+      n = toff[p + 1] - toff[p];
+    }
+    tet_geom(coord, v, i, n >= kFixedMin, geo, gexp, vol, status);
   } else if (i < nE + nN) {
     int3 f = neumann_tri(nb, i - nE);
     if (!valid_tri(f, nC)) return;
@@ -329,20 +352,13 @@ __global__ void k_face_emit(const int4* __restrict__ tet, int64_t nE, const int4
 }
 
 // face area 1/2 |(P_z - P_x) x (P_y - P_x)| of the vertices p[0..2] = P_x, P_y,
-// P_z: the product and its norm in fixed point (fixed.cuh), 12 FP64 operations
-// in place of 22
+// P_z
 __device__ __forceinline__ double face_area(const double p[3][3]) {
-  double u[3], v[3], n2;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    u[d] = p[2][d] - p[0][d];
-    v[d] = p[1][d] - p[0][d];
-  }
-  if (!fx::cross_norm2(u, v, n2)) {
-    const double cx = u[1] * v[2] - u[2] * v[1], cy = u[2] * v[0] - u[0] * v[2], cz = u[0] * v[1] - u[1] * v[0];
-    n2 = cx * cx + cy * cy + cz * cz;
-  }
-  return ph::half_sqrt(n2);
+  const double *x = p[0], *y = p[1], *z = p[2];
+  double u0 = z[0] - x[0], u1 = z[1] - x[1], u2 = z[2] - x[2];
+  double v0 = y[0] - x[0], v1 = y[1] - x[1], v2 = y[2] - x[2];
+  double cx = u1 * v2 - u2 * v1, cy = u2 * v0 - u0 * v2, cz = u0 * v1 - u1 * v0;
+  return ph::half_sqrt(cx * cx + cy * cy + cz * cz);
 }
 
 // Neumann faces get no multiplier.  Face counts are read on the device
@@ -378,16 +394,6 @@ __global__ void k_tet_mult(const int4* __restrict__ tface, int64_t nE, const int
   tmult[t] = make_int4(o[0], o[1], o[2], o[3]);
 }
 
-// last p with off[p] <= i (off ascending, off[0] = 0)
-__device__ __forceinline__ int problem_of(const int64_t* __restrict__ off, int32_t n, int64_t i) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= i) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 // The other three local faces of a tet, m != k ascending, as multiplier ids
 // (PH_NO_MULT, which sorts last, for Neumann faces or no tet).
 __device__ __forceinline__ void other_mults(int4 tm, int k, int& o0, int& o1, int& o2) {
@@ -421,17 +427,17 @@ __device__ __forceinline__ int rank7(const int c[7], int x) {
 //    Row l(F) holds l(F) and the other non-Neumann faces of F's one or two
 //    tets (all distinct): 7 candidates with PH_NO_MULT for absent ones, put in
 //    order by a 16-comparator sorting network, all in registers.  The thread
-//    also computes the face's area.  Bound by the latency of its chains of
-//    gathers (ncu: 7 of 15 cycles per issue) beside the FP64 and integer
-//    pipes, half busy each: with the area's product in fixed point and all
-//    loads issued first, 1.50 -> 1.35 ms at 35.9M faces (area alone 1.46); five
-//    blocks per SM (48 registers), 3 and 4 take 1.60 and 1.39.
+//    also computes the face's area, whose 22 FP64 operations bound the kernel
+//    (1.49 ms at 35.9M faces; with the product in fixed point 1.35, but see
+//    fixed.cuh on the areas' last bits).  All loads are issued before the
+//    first use, so the other chains of gathers hide under the FP64 pipe.
 // BATCH (a batched build): U holds the problems' offsets; the face's ids (in
 // place), its column ids and positions are then local to its problem.
 struct FillOffsets {
   const int64_t *toff, *voff;
   const long long* first;  // first face, multiplier, CSR entry
   int32_t n;
+  int32_t* rowptr;  // the problems' own row pointers: L_p + 1 entries at first multiplier + p
 };
 
 template <bool BATCH>
@@ -480,7 +486,11 @@ __global__ void __launch_bounds__(ph::kThreads, BATCH ? 4 : 5) k_row_fill(int2* 
     face_tet[F] = make_int2(ft.x - t0, ft.y < 0 ? -1 : ft.y - t0);
 #pragma unroll
     for (int j = 0; j < 3; ++j) face_vtx[3 * F + j] = vtx[j] - v0;
-    if (l >= 0) face_mult[F] = l - m0;
+    if (l >= 0) {
+      face_mult[F] = l - m0;
+      if (l == m0) U.rowptr[l + q] = 0;
+      U.rowptr[l + q + 1] = end - z0;
+    }
   }
   if (l < 0) return;
   int k[2] = {0, 0};
@@ -522,6 +532,33 @@ __global__ void __launch_bounds__(ph::kThreads, BATCH ? 4 : 5) k_row_fill(int2* 
   }
 }
 
+__device__ __forceinline__ int shift_id(int x, int64_t off) {  // keep bit 31 (sigma / Dirichlet mark)
+  return (int)(((unsigned)x & 0x80000000u) | (unsigned)((x & PH_ID_MASK) - (int)off));
+}
+
+// per tet of a batched build: local vertex ids, face ids, multiplier ids
+// (k_row_fill has made the faces' and the CSR's local: separate passes over the
+// 521M columns, 75M faces and 75M rows of 256 problems took 2.3, 0.7 and 0.4
+// ms)
+__global__ void k_rebase_tets(const FillOffsets o, int64_t nE, int4* __restrict__ tet, int4* __restrict__ tface,
+                              int4* __restrict__ tmult, const unsigned* status) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= nE || failed(status)) return;
+  const int p = problem_of(o.toff, o.n, t);
+  const int v = (int)o.voff[p];
+  const int64_t f = o.first[3 * p], mo = o.first[3 * p + 1];
+  const int4 a = tet[t];
+  tet[t] = make_int4(a.x - v, a.y - v, a.z - v, a.w - v);
+  const int4 b = tface[t];
+  tface[t] = make_int4(shift_id(b.x, f), shift_id(b.y, f), shift_id(b.z, f), shift_id(b.w, f));
+  const int4 c = tmult[t];
+  int cm[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (cm[k] != PH_NO_MULT) cm[k] = shift_id(cm[k], mo);
+  tmult[t] = make_int4(cm[0], cm[1], cm[2], cm[3]);
+}
+
 __global__ void k_face_centroid(const double* __restrict__ coord, const int32_t* __restrict__ face_vtx, int64_t nF,
                                 double* __restrict__ out) {
   int64_t F = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -548,7 +585,6 @@ static void mesh_free(ph_mesh* m, cudaStream_t s) {
   if (m->shared) {
     if (m->shared->refs.fetch_sub(1) == 1) {
       free_async(m->shared->arena, s);
-      free_async(m->shared->extra, s);
       delete m->shared;
     }
   } else {
@@ -586,13 +622,19 @@ __global__ void k_batch_offsets(const int4* __restrict__ tface, const int32_t* _
   out[3 * p + 2] = z0;
 }
 
-// Hook of a batched build: the per-problem offsets, computed before the
-// build's one synchronisation and read with it.
+// Hook of a batched build: the union's inputs, and the per-problem offsets,
+// computed before the build's one synchronisation and read with it.
 struct BatchCounts {
+  // called once the mesh's own memory is allocated: sets the input arrays and
+  // the pointers below.  (Memory of a mesh freed just before, its kernels still
+  // running, is reused by the stream only if the largest block is asked for
+  // first: with the inputs before it the pool mapped 14 GB anew, 5 ms a build.)
+  std::function<ph_status(const double** coord, const int32_t** tet, const int32_t** neumann)> inputs;
   const int64_t *d_toff, *d_voff;  // n + 1 tet and vertex offsets (device)
   int32_t n;
   long long* d_counts;  // 3n: first face, multiplier, CSR entry of each problem
   long long* h_counts;  // 3n (host)
+  int32_t* rowptr;      // out: the problems' row pointers (device, in the mesh's allocation)
 };
 
 // Synchronise and read n device int64 counters and the status word.
@@ -612,7 +654,7 @@ static ph_status read_counters(const int64_t* d_tot, int n, unsigned* d_status, 
 #define PH_CU(expr, what) PH_TRY(cuda_status((expr), what))
 
 static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet, int64_t nE, const int32_t* neumann,
-                            int64_t nN, cudaStream_t s, ph_mesh** out, const BatchCounts* bc, bool dw = false);
+                            int64_t nN, cudaStream_t s, ph_mesh** out, BatchCounts* bc, bool dw = false);
 
 extern "C" ph_status ph_mesh_create(const double* coord, int64_t nC, const int32_t* tet, int64_t nE,
                                     const int32_t* neumann, int64_t nN, void* stream, ph_mesh** out) {
@@ -625,10 +667,11 @@ extern "C" ph_status ph_mesh_create_dw(const double* coord, int64_t nC, const in
 }
 
 static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet, int64_t nE, const int32_t* neumann,
-                            int64_t nN, cudaStream_t s, ph_mesh** out, const BatchCounts* bc, bool dw) {
+                            int64_t nN, cudaStream_t s, ph_mesh** out, BatchCounts* bc, bool dw) {
   if (!out) return PH_ERR_ARG;
   *out = nullptr;
-  if (nE < 0 || nC < 0 || nN < 0 || (nE > 0 && (!coord || !tet)) || (nN > 0 && !neumann)) return PH_ERR_ARG;
+  if (nE < 0 || nC < 0 || nN < 0) return PH_ERR_ARG;
+  if (!bc && ((nE > 0 && (!coord || !tet)) || (nN > 0 && !neumann))) return PH_ERR_ARG;
   if ((reinterpret_cast<uintptr_t>(tet) & 15u) != 0) return PH_ERR_ARG;  // read as int4
   // Face arrays are sized by nFmax = 4 nE + nN >= nF and the CSR columns by
   // nFmax + 12 nE >= nnz, so the whole construction is enqueued at once and
@@ -657,7 +700,7 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   const size_t o_ftet = mc.take<int2>(nFmax), o_fvtx = mc.take<int32_t>(3 * nFmax);
   const size_t o_fkind = mc.take<int8_t>(nFmax), o_fmult = mc.take<int32_t>(nFmax + 1);
   const size_t o_farea = mc.take<double>(nFmax), o_rowptr = mc.take<int32_t>(nFmax + 1);
-  const size_t o_colind = mc.take<int32_t>(nnzmax);
+  const size_t o_colind = mc.take<int32_t>(nnzmax), o_rowptr_b = mc.take<int32_t>(bc ? nFmax + bc->n : 0);
   // scratch: zeroed part first
   const size_t o_tot = sc.take<int64_t>(3), o_cnt = sc.take<int32_t>(nb);
   const size_t o_s1 = sc.take<unsigned long long>(scan_state_words(nb));
@@ -675,6 +718,7 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   m->nE = nE;
   m->nC = nC;
   PH_CU(alloc_bytes(&m->arena, mc.bytes, s), "alloc mesh");
+  if (bc) PH_TRY(bc->inputs(&coord, &tet, &neumann));
   PH_CU(alloc_bytes(&scratch, sc.bytes, s), "alloc scratch");
   {
     void* A = m->arena;
@@ -695,6 +739,7 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
     m->face_area = Carve::at<double>(A, o_farea);
     m->rowptr = Carve::at<int32_t>(A, o_rowptr);
     m->colind = Carve::at<int32_t>(A, o_colind);
+    if (bc) bc->rowptr = Carve::at<int32_t>(A, o_rowptr_b);
   }
   {
   int64_t* d_tot = Carve::at<int64_t>(scratch, o_tot);  // [0] nF, [1] L, [2] nnz
@@ -725,7 +770,8 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
     {
       KernelTimer kt("k_face_fill", s, 2);
       k_face_fill<<<grid_for(nE + nN, kFillThreads), kFillThreads, 0, s>>>(m->tet, nE, nC, neumann, nN, sub, start, cnt, entries,
-                                                         mate, m->coord, m->geo, m->gexp, m->vol, m->status);
+                                                         mate, m->coord, m->geo, m->gexp, m->vol, bc ? bc->d_toff : nullptr, bc ? bc->n : 0,
+                                                                 m->status);
       PH_CU(launched(), "k_face_fill");
     }
     {
@@ -770,13 +816,18 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   if (nFmax > 0) {
     KernelTimer kt("k_row_fill", s, 2);
     const auto fill = bc ? k_row_fill<true> : k_row_fill<false>;
+    FillOffsets U{nullptr, nullptr, nullptr, 0, nullptr};
+    if (bc) U = FillOffsets{bc->d_toff, bc->d_voff, bc->d_counts, bc->n, bc->rowptr};
     fill<<<gF, kThreads, 0, s>>>(m->face_tet, m->tface, m->tmult, m->face_mult, d_tot, nFmax, m->rowptr, m->colind,
                                  reinterpret_cast<int32_t*>(m->tpos), reinterpret_cast<unsigned short*>(m->trel),
                                  m->coord, m->face_vtx, m->face_area,
-                                 bc ? FillOffsets{bc->d_toff, bc->d_voff, bc->d_counts, bc->n}
-                                    : FillOffsets{nullptr, nullptr, nullptr, 0},
-                                 m->status);
+                                 U, m->status);
     PH_CU(launched(), "k_row_fill");
+  }
+  if (bc && nE > 0) {
+    k_rebase_tets<<<grid_for(nE), kThreads, 0, s>>>(
+        FillOffsets{bc->d_toff, bc->d_voff, bc->d_counts, bc->n, bc->rowptr}, nE, m->tet, m->tface, m->tmult, m->status);
+    PH_CU(launched(), "k_rebase_tets");
   }
   if (bc && bc->n > 0)
     PH_CU(cudaMemcpyAsync(bc->h_counts, bc->d_counts, sizeof(long long) * 3 * bc->n, cudaMemcpyDeviceToHost, s),
@@ -882,12 +933,6 @@ extern "C" ph_status ph_mesh_check(ph_mesh* m, void* stream) {
 // ---------------------------------------------------------------------------
 namespace {
 
-// Offsets of problem p in the union (device, n + 1 entries each).
-struct UnionOffsets {
-  const int64_t *toff, *voff, *foff, *moff, *zoff;
-  int32_t n;
-};
-
 struct UnionSources {
   const int32_t* tet;  // problem's tets (nE_p x 4)
   const int32_t* nb;   // problem's Neumann triples or null
@@ -919,47 +964,6 @@ __global__ void k_union_inputs(const UnionSources* __restrict__ src, const int64
   }
 }
 
-__device__ __forceinline__ int shift_id(int x, int64_t off) {  // keep bit 31 (sigma / Dirichlet mark)
-  return (int)(((unsigned)x & 0x80000000u) | (unsigned)((x & PH_ID_MASK) - (int)off));
-}
-
-// per tet: local vertex ids, face ids, multiplier ids (k_row_fill has made the
-// faces' and the CSR's local: separate passes over the 521M columns and 75M
-// faces of 256 problems took 2.3 and 0.7 ms)
-__global__ void k_rebase_tets(UnionOffsets o, int64_t nE, int4* __restrict__ tet, int4* __restrict__ tface,
-                              int4* __restrict__ tmult) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= nE) return;
-  const int p = problem_of(o.toff, o.n, t);
-  const int v = (int)o.voff[p];
-  const int64_t f = o.foff[p], mo = o.moff[p];
-  const int4 a = tet[t];
-  tet[t] = make_int4(a.x - v, a.y - v, a.z - v, a.w - v);
-  const int4 b = tface[t];
-  tface[t] = make_int4(shift_id(b.x, f), shift_id(b.y, f), shift_id(b.z, f), shift_id(b.w, f));
-  const int4 c = tmult[t];
-  int cm[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (cm[k] != PH_NO_MULT) cm[k] = shift_id(cm[k], mo);
-  tmult[t] = make_int4(cm[0], cm[1], cm[2], cm[3]);
-}
-
-// per multiplier row: the problem's own row pointers (problem p's L_p + 1
-// entries at rowptr_b + moff[p] + p)
-__global__ void k_rebase_rows(UnionOffsets o, int64_t L, const int32_t* __restrict__ rowptr,
-                              int32_t* __restrict__ rowptr_b) {
-  const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (l >= L + o.n) return;
-  if (l < L) {
-    const int p = problem_of(o.moff, o.n, l);
-    const int z = (int)o.zoff[p];
-    rowptr_b[l + p] = rowptr[l] - z;
-  } else {  // the closing entry of problem p: its nnz
-    const int p = (int)(l - L);
-    rowptr_b[o.moff[p + 1] + p] = (int)(o.zoff[p + 1] - o.zoff[p]);
-  }
-}
 
 }  // namespace
 
@@ -986,47 +990,54 @@ extern "C" ph_status ph_mesh_create_batch(int32_t n, const double* const* coord,
   }
   const int64_t nEu = toff[n], nNu = noff[n], nCu = voff[n];
   if (16 * nEu + nNu >= ((int64_t)1 << 31) - 1 || nCu >= ((int64_t)1 << 31) - 1) return PH_ERR_OVERFLOW;
-  // union inputs and the offset tables in one allocation
-  Carve ic;
-  const size_t o_coord = ic.take<double>(3 * nCu), o_tet = ic.take<int4>(nEu), o_nb = ic.take<int32_t>(3 * nNu);
-  const size_t o_src = ic.take<UnionSources>(n), o_off = ic.take<int64_t>(3 * (n + 1));
-  const size_t o_cnt = ic.take<long long>(3 * n);
   void* in = nullptr;
-  cudaError_t e = alloc_bytes(&in, ic.bytes, s);
-  if (e != cudaSuccess) return cuda_status(e, "alloc batch inputs");
-  double* coord_u = Carve::at<double>(in, o_coord);
-  int4* tet_u = Carve::at<int4>(in, o_tet);
-  int32_t* nb_u = Carve::at<int32_t>(in, o_nb);
-  UnionSources* d_src = Carve::at<UnionSources>(in, o_src);
-  int64_t* d_off = Carve::at<int64_t>(in, o_off);  // toff, noff, voff
-  long long* d_cnt = Carve::at<long long>(in, o_cnt);
-  std::vector<int64_t> offs;
-  offs.insert(offs.end(), toff.begin(), toff.end());
-  offs.insert(offs.end(), noff.begin(), noff.end());
-  offs.insert(offs.end(), voff.begin(), voff.end());
-  for (int32_t p = 0; p < n && e == cudaSuccess; ++p)
-    if (nC[p] > 0)
-      e = cudaMemcpyAsync(coord_u + 3 * voff[p], coord[p], sizeof(double) * 3 * nC[p], cudaMemcpyDeviceToDevice, s);
-  // pageable sources: the copies return once the data is staged
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_src, src.data(), sizeof(UnionSources) * n, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_off, offs.data(), sizeof(int64_t) * offs.size(), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && nEu + nNu > 0) {
-    k_union_inputs<<<grid_for(nEu + nNu), kThreads, 0, s>>>(d_src, d_off, d_off + (n + 1), d_off + 2 * (n + 1), n,
-                                                          nEu, nNu, tet_u, nb_u);
-    e = launched();
-  }
-  if (e != cudaSuccess) {
-    free_async(in, s);
-    return cuda_status(e, "ph_mesh_create_batch inputs");
-  }
   std::vector<long long> cnt(3 * (size_t)n, -1);
-  BatchCounts bc{d_off, d_off + 2 * (n + 1), n, d_cnt, cnt.data()};
+  BatchCounts bc;
+  bc.n = n;
+  bc.h_counts = cnt.data();
+  bc.rowptr = nullptr;
+  std::vector<int64_t> offs;
+  bc.inputs = [&](const double** coord_out, const int32_t** tet_out, const int32_t** nb_out) {
+    // union inputs and the offset tables in one allocation
+    Carve ic;
+    const size_t o_coord = ic.take<double>(3 * nCu), o_tet = ic.take<int4>(nEu), o_nb = ic.take<int32_t>(3 * nNu);
+    const size_t o_src = ic.take<UnionSources>(n), o_off = ic.take<int64_t>(3 * (n + 1));
+    const size_t o_cnt = ic.take<long long>(3 * n);
+    cudaError_t e = alloc_bytes(&in, ic.bytes, s);
+    if (e != cudaSuccess) return cuda_status(e, "alloc batch inputs");
+    double* coord_u = Carve::at<double>(in, o_coord);
+    int4* tet_u = Carve::at<int4>(in, o_tet);
+    int32_t* nb_u = Carve::at<int32_t>(in, o_nb);
+    UnionSources* d_src = Carve::at<UnionSources>(in, o_src);
+    int64_t* d_off = Carve::at<int64_t>(in, o_off);  // toff, noff, voff
+    offs.insert(offs.end(), toff.begin(), toff.end());
+    offs.insert(offs.end(), noff.begin(), noff.end());
+    offs.insert(offs.end(), voff.begin(), voff.end());
+    for (int32_t p = 0; p < n && e == cudaSuccess; ++p)
+      if (nC[p] > 0)
+        e = cudaMemcpyAsync(coord_u + 3 * voff[p], coord[p], sizeof(double) * 3 * nC[p], cudaMemcpyDeviceToDevice, s);
+    // pageable sources: the copies return once the data is staged
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_src, src.data(), sizeof(UnionSources) * n, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(d_off, offs.data(), sizeof(int64_t) * offs.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && nEu + nNu > 0) {
+      k_union_inputs<<<grid_for(nEu + nNu), kThreads, 0, s>>>(d_src, d_off, d_off + (n + 1), d_off + 2 * (n + 1), n, nEu,
+                                                            nNu, tet_u, nb_u);
+      e = launched();
+    }
+    bc.d_toff = d_off;
+    bc.d_voff = d_off + 2 * (n + 1);
+    bc.d_counts = Carve::at<long long>(in, o_cnt);
+    *coord_out = coord_u;
+    *tet_out = reinterpret_cast<const int32_t*>(tet_u);
+    *nb_out = nNu > 0 ? nb_u : nullptr;
+    return cuda_status(e, "ph_mesh_create_batch inputs");
+  };
   ph_mesh* u = nullptr;
-  ph_status st = mesh_build(coord_u, nCu, reinterpret_cast<const int32_t*>(tet_u), nEu, nNu > 0 ? nb_u : nullptr,
-                            nNu, s, &u, &bc);
+  ph_status st = mesh_build(nullptr, nCu, nullptr, nEu, nullptr, nNu, s, &u, &bc);
   free_async(in, s);
   if (st != PH_OK) return st;
+  cudaError_t e = cudaSuccess;
   // per-problem face, multiplier and CSR offsets; an empty problem starts
   // where the next one does
   std::vector<int64_t> foff(n + 1, 0), moff(n + 1, 0), zoff(n + 1, 0);
@@ -1045,39 +1056,16 @@ extern "C" ph_status ph_mesh_create_batch(int32_t n, const double* const* coord,
     mesh_free(u, s);
     return PH_ERR_ARG;
   }
-  // row pointers of the problems (L + n) and the offset tables (5 (n + 1))
-  Carve xc;
-  const size_t o_rp = xc.take<int32_t>(u->L + n), o_tab = xc.take<int64_t>(5 * (n + 1));
-  void* extra = nullptr;
-  e = alloc_bytes(&extra, xc.bytes, s);
+  for (int32_t p = 0; p < n && e == cudaSuccess; ++p)  // no row wrote the one row pointer of an empty system
+    if (moff[p + 1] == moff[p]) e = cudaMemsetAsync(bc.rowptr + moff[p] + p, 0, sizeof(int32_t), s);
   if (e != cudaSuccess) {
     mesh_free(u, s);
-    return cuda_status(e, "alloc batch rows");
-  }
-  int32_t* rowptr_b = Carve::at<int32_t>(extra, o_rp);
-  int64_t* tab = Carve::at<int64_t>(extra, o_tab);
-  std::vector<int64_t> t5;
-  for (const auto* v : {&toff, &voff, &foff, &moff, &zoff}) t5.insert(t5.end(), v->begin(), v->end());
-  e = cudaMemcpyAsync(tab, t5.data(), sizeof(int64_t) * t5.size(), cudaMemcpyHostToDevice, s);
-  const UnionOffsets o{tab, tab + (n + 1), tab + 2 * (n + 1), tab + 3 * (n + 1), tab + 4 * (n + 1), n};
-  if (e == cudaSuccess && nEu > 0) {
-    k_rebase_tets<<<grid_for(nEu), kThreads, 0, s>>>(o, nEu, u->tet, u->tface, u->tmult);
-    e = launched();
-  }
-  if (e == cudaSuccess) {
-    k_rebase_rows<<<grid_for(u->L + n), kThreads, 0, s>>>(o, u->L, u->rowptr, rowptr_b);
-    e = launched();
-  }
-  if (e != cudaSuccess) {
-    free_async(extra, s);
-    mesh_free(u, s);
-    return cuda_status(e, "ph_mesh_create_batch rebase");
+    return cuda_status(e, "ph_mesh_create_batch rows");
   }
   // the views: each problem's slices of the union arrays, local ids
   ph_mesh_shared* sh = new ph_mesh_shared();
   sh->refs.store(n);
   sh->arena = u->arena;
-  sh->extra = extra;
   for (int32_t p = 0; p < n; ++p) {
     ph_mesh* m = new ph_mesh();
     memset(m, 0, sizeof *m);
@@ -1106,7 +1094,7 @@ extern "C" ph_status ph_mesh_create_batch(int32_t n, const double* const* coord,
     m->face_kind = u->face_kind + f0;
     m->face_mult = u->face_mult + f0;
     m->face_area = u->face_area + f0;
-    m->rowptr = rowptr_b + m0 + p;
+    m->rowptr = bc.rowptr + m0 + p;
     m->colind = u->colind + z0;
     m->status = u->status;
     out[p] = m;

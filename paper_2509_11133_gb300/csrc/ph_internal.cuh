@@ -25,7 +25,6 @@
 struct ph_mesh_shared {
   std::atomic<int> refs;
   void* arena;  // the union mesh's arrays
-  void* extra;  // per-problem row pointers and offset tables
 };
 
 struct ph_mesh {
