@@ -119,10 +119,9 @@ __device__ __forceinline__ int problem_of(const int64_t* __restrict__ off, int32
 }
 
 // 1. histogram of face keys by bucket
-__global__ void k_face_count(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
+__device__ __forceinline__ void face_count_item(int64_t i, const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
                              int64_t nN, int sub, int32_t* __restrict__ cnt, int4* __restrict__ tet_copy,
                              unsigned* status) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < nE) {
     int4 v = tet[i];
     tet_copy[i] = v;  // the mesh's own copy of the input
@@ -136,6 +135,13 @@ __global__ void k_face_count(const int4* __restrict__ tet, int64_t nE, int64_t n
   }
 }
 
+__global__ void k_face_count(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
+                             int64_t nN, int sub, int32_t* __restrict__ cnt, int4* __restrict__ tet_copy,
+                             unsigned* status) {
+  face_count_item(blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+      tet, nE, nC, nb, nN, sub, cnt, tet_copy, status);
+}
+
 // 2. scatter keys into buckets: entry = (v0, v1, v2, slot), slot = 4t+k for
 //    tet faces and 4nE+i for Neumann triples.  cnt counts down to 0.  The
 //    same thread then computes the tet's geometry: G_e in fixed point on the
@@ -146,12 +152,12 @@ __global__ void k_face_count(const int4* __restrict__ tet, int64_t nE, int64_t n
 //    at 96 registers 1.63; storing the entries after the geometry instead of
 //    before it holds their stores back, 1.26.
 constexpr int kFillThreads = 128;
-__global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
+template <bool GEO>
+__device__ __forceinline__ void face_fill_item(int64_t i, const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
                             int64_t nN, int sub, const int32_t* __restrict__ start, int32_t* __restrict__ cnt,
                             int4* __restrict__ entries, int32_t* __restrict__ mate, const double* __restrict__ coord,
                             double* __restrict__ geo, int32_t* __restrict__ gexp, double2* __restrict__ vol,
                             const int64_t* __restrict__ toff, int32_t nprob, unsigned* status) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (failed(status)) return;
   if (i < nE) {
     int4 v = tet[i];
@@ -168,6 +174,7 @@ __global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __res
       entries[pos[k]] = make_int4(s.x, s.y, s.z, (int)(4 * i + k));
     }
     reinterpret_cast<int4*>(mate)[i] = make_int4(-1, -1, -1, -1);  // no mate yet (boundary)
+    if (!GEO) return;
     int64_t n = nE;  // tets of the tet's mesh
     if (toff) {
       const int p = problem_of(toff, nprob, i);
@@ -182,6 +189,16 @@ __global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __res
     int pos = start[b] + atomicSub(&cnt[b], 1) - 1;
     entries[pos] = make_int4(s.x, s.y, s.z, (int)i + 3 * (int)nE);  // slot 4nE + (i - nE)
   }
+}
+
+template <bool GEO>
+__global__ void __launch_bounds__(kFillThreads, 6) k_face_fill(const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
+                            int64_t nN, int sub, const int32_t* __restrict__ start, int32_t* __restrict__ cnt,
+                            int4* __restrict__ entries, int32_t* __restrict__ mate, const double* __restrict__ coord,
+                            double* __restrict__ geo, int32_t* __restrict__ gexp, double2* __restrict__ vol,
+                            const int64_t* __restrict__ toff, int32_t nprob, unsigned* status) {
+  face_fill_item<GEO>(blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+      tet, nE, nC, nb, nN, sub, start, cnt, entries, mate, coord, geo, gexp, vol, toff, nprob, status);
 }
 
 // Outcome of one entry's scan: a tet entry records its mate (and its mate's
@@ -220,10 +237,9 @@ __device__ __forceinline__ void count_match(int4 k, int4 e, int ntet, int& nt, i
 //    of loads in flight per thread.  The kernel issues instructions at close
 //    to the SM's rate, so the loop carries no more than the loads and
 //    compares; the bucket hash keeps the scans short.
-__global__ void k_face_match(const int4* __restrict__ entries, int64_t nent, const int32_t* __restrict__ start,
+__device__ __forceinline__ void face_match_item(int64_t i0, const int4* __restrict__ entries, int64_t nent, const int32_t* __restrict__ start,
                              int sub, int64_t nE, int32_t* __restrict__ mate, unsigned* status) {
   const int64_t half = (nent + 1) >> 1;
-  const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i0 >= half || failed(status)) return;
   const int64_t i1 = i0 + half;
   const bool has1 = i1 < nent;
@@ -249,6 +265,12 @@ __global__ void k_face_match(const int4* __restrict__ entries, int64_t nent, con
   }
   settle_entry(e0, ntet, nt0, nn0, tm0, mate, status);
   if (has1) settle_entry(e1, ntet, nt1, nn1, tm1, mate, status);
+}
+
+__global__ void k_face_match(const int4* __restrict__ entries, int64_t nent, const int32_t* __restrict__ start,
+                             int sub, int64_t nE, int32_t* __restrict__ mate, unsigned* status) {
+  face_match_item(blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+      entries, nent, start, sub, nE, mate, status);
 }
 
 // 4. face bases: an exclusive scan of the number of first occurrences per tet,
@@ -326,13 +348,12 @@ __device__ __forceinline__ void load_owners(int64_t t, int4 m, const int4* __res
 //    per tet of the face (7 interior, 4 boundary); k_tet_mult is not needed.
 //    Each thread takes two tets, t and t + half, and issues all their loads
 //    before using any (its warps mostly wait on loads).
-__global__ void k_face_emit(const int4* __restrict__ tet, int64_t nE, const int4* __restrict__ mate4,
+__device__ __forceinline__ void face_emit_item(int64_t t0, const int4* __restrict__ tet, int64_t nE, const int4* __restrict__ mate4,
                             const int32_t* __restrict__ fbase, int4* __restrict__ tface, int2* __restrict__ face_tet,
                             int32_t* __restrict__ face_vtx, int8_t* __restrict__ face_kind,
                             int32_t* __restrict__ flag, int32_t* __restrict__ mult_iota, int4* __restrict__ tmult,
                             int32_t* __restrict__ rowlen, const unsigned* status) {
   const int64_t half = (nE + 1) >> 1;
-  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t0 >= half || failed(status)) return;
   const int64_t t1 = t0 + half;
   const bool has1 = t1 < nE;
@@ -351,6 +372,15 @@ __global__ void k_face_emit(const int4* __restrict__ tet, int64_t nE, const int4
     emit_tet(t1, v1, m1, fb1, om1, ofb1, nF, tface, face_tet, face_vtx, face_kind, flag, mult_iota, tmult, rowlen);
 }
 
+__global__ void k_face_emit(const int4* __restrict__ tet, int64_t nE, const int4* __restrict__ mate4,
+                            const int32_t* __restrict__ fbase, int4* __restrict__ tface, int2* __restrict__ face_tet,
+                            int32_t* __restrict__ face_vtx, int8_t* __restrict__ face_kind,
+                            int32_t* __restrict__ flag, int32_t* __restrict__ mult_iota, int4* __restrict__ tmult,
+                            int32_t* __restrict__ rowlen, const unsigned* status) {
+  face_emit_item(blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+      tet, nE, mate4, fbase, tface, face_tet, face_vtx, face_kind, flag, mult_iota, tmult, rowlen, status);
+}
+
 // face area 1/2 |(P_z - P_x) x (P_y - P_x)| of the vertices p[0..2] = P_x, P_y,
 // P_z
 __device__ __forceinline__ double face_area(const double p[3][3]) {
@@ -363,19 +393,23 @@ __device__ __forceinline__ double face_area(const double p[3][3]) {
 
 // Neumann faces get no multiplier.  Face counts are read on the device
 // (d_tot[0] = nF), the grid covers the upper bound.
-__global__ void k_mult_fix(int32_t* __restrict__ face_mult, const int8_t* __restrict__ face_kind,
+__device__ __forceinline__ void mult_fix_item(int64_t F, int32_t* __restrict__ face_mult, const int8_t* __restrict__ face_kind,
                            const int64_t* __restrict__ d_tot, int64_t nFmax, const unsigned* status) {
-  int64_t F = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (F >= nFmax || F >= d_tot[0] || failed(status)) return;
   if (face_kind[F] == 2) face_mult[F] = -1;
 }
 
+__global__ void k_mult_fix(int32_t* __restrict__ face_mult, const int8_t* __restrict__ face_kind,
+                           const int64_t* __restrict__ d_tot, int64_t nFmax, const unsigned* status) {
+  mult_fix_item(blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+      face_mult, face_kind, d_tot, nFmax, status);
+}
+
 // 7. per-slot multiplier ids and row lengths: row l(F) = 1 + sum over F's
 //    tets of (non-Neumann faces of the tet) - 1.
-__global__ void k_tet_mult(const int4* __restrict__ tface, int64_t nE, const int32_t* __restrict__ face_mult,
+__device__ __forceinline__ void tet_mult_item(int64_t t, const int4* __restrict__ tface, int64_t nE, const int32_t* __restrict__ face_mult,
                            const int2* __restrict__ face_tet, int4* __restrict__ tmult, int32_t* __restrict__ rowlen,
                            const unsigned* status) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE || failed(status)) return;
   int4 tf = tface[t];
   int l[4], o[4];
@@ -392,6 +426,13 @@ __global__ void k_tet_mult(const int4* __restrict__ tface, int64_t nE, const int
   for (int k = 0; k < 4; ++k)
     if (l[k] >= 0) atomicAdd(&rowlen[l[k]], mT - 1 + (comp(tf, k) >= 0 ? 1 : 0));
   tmult[t] = make_int4(o[0], o[1], o[2], o[3]);
+}
+
+__global__ void k_tet_mult(const int4* __restrict__ tface, int64_t nE, const int32_t* __restrict__ face_mult,
+                           const int2* __restrict__ face_tet, int4* __restrict__ tmult, int32_t* __restrict__ rowlen,
+                           const unsigned* status) {
+  tet_mult_item(blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+      tface, nE, face_mult, face_tet, tmult, rowlen, status);
 }
 
 // The other three local faces of a tet, m != k ascending, as multiplier ids
@@ -422,8 +463,9 @@ __device__ __forceinline__ int rank7(const int c[7], int x) {
   return r;
 }
 
-// 8. column indices of each row (ascending) and each slot's scatter positions: tpos = diagonal, trel = rank offsets of the
-//    other three local faces (4-bit two's complement, m != k ascending).
+// 8. column indices of each row (ascending) and each slot's scatter positions:
+//    tpos = diagonal, trel = rank offsets of the other three local faces (4-bit
+//    two's complement, m != k ascending).
 //    Row l(F) holds l(F) and the other non-Neumann faces of F's one or two
 //    tets (all distinct): 7 candidates with PH_NO_MULT for absent ones, put in
 //    order by a 16-comparator sorting network, all in registers.  The thread
@@ -440,8 +482,8 @@ struct FillOffsets {
   int32_t* rowptr;  // the problems' own row pointers: L_p + 1 entries at first multiplier + p
 };
 
-template <bool BATCH>
-__global__ void __launch_bounds__(ph::kThreads, BATCH ? 4 : 5) k_row_fill(int2* __restrict__ face_tet, const int4* __restrict__ tface,
+template <bool BATCH, bool AREA>
+__device__ __forceinline__ void row_fill_item(int64_t F, int2* __restrict__ face_tet, const int4* __restrict__ tface,
                            const int4* __restrict__ tmult, int32_t* __restrict__ face_mult,
                            const int64_t* __restrict__ d_tot, int64_t nFmax,
                            const int32_t* __restrict__ rowptr, int32_t* __restrict__ colind,
@@ -449,7 +491,6 @@ __global__ void __launch_bounds__(ph::kThreads, BATCH ? 4 : 5) k_row_fill(int2* 
                            unsigned short* __restrict__ trel, const double* __restrict__ coord,
                            int32_t* __restrict__ face_vtx, double* __restrict__ area, const FillOffsets U,
                            unsigned* status) {
-  const int64_t F = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (F >= nFmax || F >= d_tot[0] || failed(status)) return;
   // every load whose address is known, before anything uses one: the vertices'
   // and the tets' chains of loads run side by side
@@ -467,16 +508,17 @@ __global__ void __launch_bounds__(ph::kThreads, BATCH ? 4 : 5) k_row_fill(int2* 
       tm[side] = tmult[T[side]];
     }
   double p[3][3];
+  if (AREA)
 #pragma unroll
-  for (int j = 0; j < 3; ++j)
+    for (int j = 0; j < 3; ++j)
 #pragma unroll
-    for (int d = 0; d < 3; ++d) p[j][d] = coord[3 * (int64_t)vtx[j] + d];
+      for (int d = 0; d < 3; ++d) p[j][d] = coord[3 * (int64_t)vtx[j] + d];
   int base = 0, end = 0;
   if (l >= 0) {
     base = rowptr[l];
     end = rowptr[l + 1];
   }
-  area[F] = face_area(p);
+  if (AREA) area[F] = face_area(p);
   int m0 = 0, z0 = 0;
   if (BATCH) {
     const int q = problem_of(U.toff, U.n, T[0]);
@@ -530,6 +572,161 @@ __global__ void __launch_bounds__(ph::kThreads, BATCH ? 4 : 5) k_row_fill(int2* 
     tpos[4 * (int64_t)T[side] + k[side]] = diag;
     trel[4 * (int64_t)T[side] + k[side]] = (unsigned short)bits;
   }
+}
+
+template <bool BATCH, bool AREA>
+__global__ void __launch_bounds__(ph::kThreads, BATCH ? 4 : 5) k_row_fill(int2* __restrict__ face_tet, const int4* __restrict__ tface,
+                           const int4* __restrict__ tmult, int32_t* __restrict__ face_mult,
+                           const int64_t* __restrict__ d_tot, int64_t nFmax,
+                           const int32_t* __restrict__ rowptr, int32_t* __restrict__ colind,
+                           int32_t* __restrict__ tpos,
+                           unsigned short* __restrict__ trel, const double* __restrict__ coord,
+                           int32_t* __restrict__ face_vtx, double* __restrict__ area, const FillOffsets U,
+                           unsigned* status) {
+  row_fill_item<BATCH, AREA>(blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+      face_tet, tface, tmult, face_mult, d_tot, nFmax, rowptr, colind, tpos, trel, coord, face_vtx, area, U, status);
+}
+
+
+// ---------------------------------------------------------------------------
+// Small meshes: the connectivity in one launch of one block, the geometry in
+// another.  The nine launches above take 2.5 to 8 us each whatever they do (~60
+// us with their gaps at 864 tets); here a phase costs its chain of L1 and L2
+// trips.  The items are the kernels' own, so the result is theirs bit for bit.
+// One block: a cluster would need the scans across its blocks, and the FP64
+// work (97 operations per tet, 13 us on one SM at 864 tets) is what wants
+// spreading, which k_small_geom does.
+// ---------------------------------------------------------------------------
+constexpr int kSmallThreads = 1024;
+constexpr int64_t kSmallTets = 1536, kSmallBuckets = 8192;
+
+struct SmallMesh {
+  const int4* tet_in;
+  const double* coord_in;
+  const int32_t* nb;
+  int64_t nE, nC, nN;
+  int sub;
+  int64_t nbuckets;
+  int32_t *cnt, *start, *newc, *flag, *rowlen;
+  int4* entries;
+  int32_t* mate;
+  int64_t* d_tot;
+  // the mesh's arrays
+  double* coord;
+  int4 *tet, *tface, *tmult;
+  int2* face_tet;
+  int32_t *face_vtx, *face_mult, *rowptr, *colind, *tpos;
+  int8_t* face_kind;
+  unsigned short* trel;
+  double *geo, *face_area;
+  int32_t* gexp;
+  double2* vol;
+  unsigned* status;
+};
+
+// Exclusive prefix sum of n values of in(i) into out, total returned, by the
+// whole block (each thread a run of consecutive values).
+template <class F>
+__device__ __forceinline__ int small_scan(int64_t n, const F& in, int32_t* out) {
+  __shared__ int warp_sum[kSmallThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int64_t per = (n + kSmallThreads - 1) / kSmallThreads, lo = min(n, tid * per), hi = min(n, lo + per);
+  int sum = 0;
+  for (int64_t i = lo; i < hi; ++i) sum += in(i);
+  int inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += u;
+  }
+  if (lane == 31) warp_sum[wid] = inc;
+  __syncthreads();
+  if (wid == 0) {
+    int w = warp_sum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += u;
+    }
+    warp_sum[lane] = w;
+  }
+  __syncthreads();
+  const int total = warp_sum[kSmallThreads / 32 - 1];
+  int run = inc - sum + (wid > 0 ? warp_sum[wid - 1] : 0);
+  for (int64_t i = lo; i < hi; ++i) {
+    const int v = in(i);  // out may be in's array: read before it is written
+    out[i] = run;
+    run += v;
+  }
+  __syncthreads();
+  return total;
+}
+
+__global__ void __launch_bounds__(kSmallThreads) k_small_connect(const SmallMesh m) {
+  const int tid = threadIdx.x;
+  const int64_t nE = m.nE, nN = m.nN, nF4 = 4 * nE + nN;
+  if (tid == 0) *m.status = 0;
+  for (int64_t i = tid; i < m.nbuckets; i += kSmallThreads) m.cnt[i] = 0;
+  for (int64_t i = tid; i < 3 * m.nC; i += kSmallThreads) m.coord[i] = m.coord_in[i];
+  if (nN > 0)
+    for (int64_t i = tid; i <= nF4; i += kSmallThreads) m.flag[i] = m.rowlen[i] = 0;
+  __syncthreads();
+  for (int64_t i = tid; i < nE + nN; i += kSmallThreads)
+    face_count_item(i, m.tet_in, nE, m.nC, m.nb, nN, m.sub, m.cnt, m.tet, m.status);
+  __syncthreads();
+  small_scan(m.nbuckets, [&](int64_t i) { return m.cnt[i]; }, m.start);
+  for (int64_t i = tid; i < nE + nN; i += kSmallThreads)
+    face_fill_item<false>(i, m.tet, nE, m.nC, m.nb, nN, m.sub, m.start, m.cnt, m.entries, m.mate, nullptr, nullptr,
+                          nullptr, nullptr, nullptr, 0, m.status);
+  __syncthreads();
+  for (int64_t i = tid; i < (nF4 + 1) / 2; i += kSmallThreads)
+    face_match_item(i, m.entries, nF4, m.start, m.sub, nE, m.mate, m.status);
+  __syncthreads();
+  const int4* mate4 = reinterpret_cast<const int4*>(m.mate);
+  const int nF = small_scan(nE + 1, [&](int64_t i) { return i < nE ? ph::first_occurrences(mate4[i], (int)(4 * i)) : 0; },
+                            m.newc);
+  if (tid == 0) m.d_tot[0] = nF;
+  for (int64_t i = tid; i < (nE + 1) / 2; i += kSmallThreads)
+    face_emit_item(i, m.tet, nE, mate4, m.newc, m.tface, m.face_tet, m.face_vtx, m.face_kind, nN > 0 ? m.flag : nullptr,
+                   nN > 0 ? nullptr : m.face_mult, m.tmult, m.rowlen, m.status);
+  __syncthreads();
+  int L = nF;
+  if (nN > 0) {
+    L = small_scan(nF + 1, [&](int64_t i) { return m.flag[i]; }, m.face_mult);
+    for (int64_t F = tid; F < nF; F += kSmallThreads)
+      mult_fix_item(F, m.face_mult, m.face_kind, m.d_tot, nF4, m.status);
+    __syncthreads();
+    for (int64_t t = tid; t < nE; t += kSmallThreads)
+      tet_mult_item(t, m.tface, nE, m.face_mult, m.face_tet, m.tmult, m.rowlen, m.status);
+    __syncthreads();
+  }
+  const int nnz = small_scan(L + 1, [&](int64_t i) { return m.rowlen[i]; }, m.rowptr);
+  if (tid == 0) {
+    m.d_tot[1] = L;
+    m.d_tot[2] = nnz;
+  }
+  const FillOffsets none{nullptr, nullptr, nullptr, 0, nullptr};
+  for (int64_t F = tid; F < nF; F += kSmallThreads)
+    row_fill_item<false, false>(F, m.face_tet, m.tface, m.tmult, m.face_mult, m.d_tot, nF4, m.rowptr, m.colind, m.tpos,
+                                m.trel, m.coord, m.face_vtx, m.face_area, none, m.status);
+}
+
+// The geometry of tet i < nE, or the area of face i - nE.
+__global__ void __launch_bounds__(128) k_small_geom(const SmallMesh m) {
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (failed(m.status)) return;
+  if (i < m.nE) {
+    tet_geom(m.coord, m.tet[i], i, m.nE >= kFixedMin, m.geo, m.gexp, m.vol, m.status);
+    return;
+  }
+  i -= m.nE;
+  if (i >= m.d_tot[0]) return;
+  double p[3][3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) p[j][d] = m.coord[3 * (int64_t)m.face_vtx[3 * i + j] + d];
+  m.face_area[i] = face_area(p);
 }
 
 __device__ __forceinline__ int shift_id(int x, int64_t off) {  // keep bit 31 (sigma / Dirichlet mark)
@@ -754,6 +951,18 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   unsigned long long* st2 = Carve::at<unsigned long long>(scratch, o_s2);
   unsigned long long* st3 = Carve::at<unsigned long long>(scratch, o_s3);
   unsigned long long* st4 = Carve::at<unsigned long long>(scratch, o_s4);
+  if (!bc && nE > 0 && nE <= kSmallTets && nb <= kSmallBuckets && nN <= 4 * nE) {
+    const SmallMesh sm{reinterpret_cast<const int4*>(tet), coord, neumann, nE, nC, nN, sub, nb, cnt, start, newc, flag,
+                       rowlen, entries, mate, d_tot, m->coord, m->tet, m->tface, m->tmult, m->face_tet, m->face_vtx,
+                       m->face_mult, m->rowptr, m->colind, reinterpret_cast<int32_t*>(m->tpos), m->face_kind,
+                       reinterpret_cast<unsigned short*>(m->trel), m->geo, m->face_area, m->gexp, m->vol, m->status};
+    k_small_connect<<<1, kSmallThreads, 0, s>>>(sm);
+    PH_CU(launched(), "k_small_connect");
+    k_small_geom<<<grid_for(nE + nFmax, 128), 128, 0, s>>>(sm);
+    PH_CU(launched(), "k_small_geom");
+    PH_TRY(read_counters(d_tot, 3, m->status, s, tot, &bits));
+    goto built;
+  }
   PH_CU(cudaMemsetAsync(scratch, 0, zero_bytes, s), "memset");
   PH_CU(cudaMemsetAsync(m->status, 0, sizeof(unsigned), s), "memset");
   if (nC > 0) PH_CU(cudaMemcpyAsync(m->coord, coord, sizeof(double) * 3 * nC, cudaMemcpyDeviceToDevice, s), "copy");
@@ -769,7 +978,7 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   if (nent > 0) {
     {
       KernelTimer kt("k_face_fill", s, 2);
-      k_face_fill<<<grid_for(nE + nN, kFillThreads), kFillThreads, 0, s>>>(m->tet, nE, nC, neumann, nN, sub, start, cnt, entries,
+      k_face_fill<true><<<grid_for(nE + nN, kFillThreads), kFillThreads, 0, s>>>(m->tet, nE, nC, neumann, nN, sub, start, cnt, entries,
                                                          mate, m->coord, m->geo, m->gexp, m->vol, bc ? bc->d_toff : nullptr, bc ? bc->n : 0,
                                                                  m->status);
       PH_CU(launched(), "k_face_fill");
@@ -815,7 +1024,7 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   // --- CSR columns and scatter positions (slots without a multiplier are never read)
   if (nFmax > 0) {
     KernelTimer kt("k_row_fill", s, 2);
-    const auto fill = bc ? k_row_fill<true> : k_row_fill<false>;
+    const auto fill = bc ? k_row_fill<true, true> : k_row_fill<false, true>;
     FillOffsets U{nullptr, nullptr, nullptr, 0, nullptr};
     if (bc) U = FillOffsets{bc->d_toff, bc->d_voff, bc->d_counts, bc->n, bc->rowptr};
     fill<<<gF, kThreads, 0, s>>>(m->face_tet, m->tface, m->tmult, m->face_mult, d_tot, nFmax, m->rowptr, m->colind,
@@ -835,6 +1044,7 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
   // the one synchronisation: counts and the first error of any kernel
   PH_TRY(read_counters(d_tot, 3, m->status, s, tot, &bits));
   }
+built:
   free_async(scratch, s);
   scratch = nullptr;
   if (bits) { st = status_from_bits(bits); goto fail; }
