@@ -98,16 +98,6 @@ __device__ __forceinline__ void tet_geom(const double* __restrict__ coord, int4 
   vol[t] = make_double2(adet, rdet);
 }
 
-// Meshes of at least so many tets get the fixed-point record (fixed.cuh), smaller
-// ones the fp64 record.  The two differ in the last bits of Q, which an
-// unconverged Jacobi solve (7,000 iterations at 23,328 tets, rtol 1e-10) turns
-// into 4e-9 of Lambda: systems of the size that is solved that way keep their
-// bits.  There the FP64 pipe is not yet the bound: fixed point takes 9.7 us for
-// 11.8 of k_assemble at 16,464 tets, 13.8 for 16.2 at 34,992, 22 for 31 at
-// 95,832, 49 for 82 at 296,352; k_face_fill 8.5 for 8.6, 9.6 for 10.2, 13.5
-// for 15.9, 23 for 31.
-constexpr int64_t kFixedMin = 32768;
-
 // last p with off[p] <= i (off ascending, off[0] = 0)
 __device__ __forceinline__ int problem_of(const int64_t* __restrict__ off, int32_t n, int64_t i) {
   int lo = 0, hi = n - 1;
@@ -180,7 +170,7 @@ __device__ __forceinline__ void face_fill_item(int64_t i, const int4* __restrict
       const int p = problem_of(toff, nprob, i);
       n = toff[p + 1] - toff[p];
     }
-    tet_geom(coord, v, i, n >= kFixedMin, geo, gexp, vol, status);
+    tet_geom(coord, v, i, n >= ph::kFixedMin, geo, gexp, vol, status);
   } else if (i < nE + nN) {
     int3 f = neumann_tri(nb, i - nE);
     if (!valid_tri(f, nC)) return;
@@ -285,13 +275,13 @@ __device__ __forceinline__ int first_rank(int4 m, int s0, int k) {
   return r;
 }
 
-// Outputs of tet t, given its tuple v, mates m, face base fb and, for each
-// face it does not own, its owner's mates om[k] and face base ofb[k].
+// Face ids of tet t, given its tuple v, mates m, face base fb and, for each face
+// it does not own, its owner's mates om[k] and face base ofb[k]; own(F, T-,
+// tuple, kind) takes each face it owns (a first occurrence).  With tmult (no
+// Neumann faces) also the slots' multiplier ids, l(F) = F.
+template <class Own>
 __device__ __forceinline__ void emit_tet(int64_t t, int4 v, int4 m, int fb, const int4 om[4], const int ofb[4],
-                                         int64_t nF, int4* __restrict__ tface, int2* __restrict__ face_tet,
-                                         int32_t* __restrict__ face_vtx, int8_t* __restrict__ face_kind,
-                                         int32_t* __restrict__ flag, int32_t* __restrict__ mult_iota,
-                                         int4* __restrict__ tmult, int32_t* __restrict__ rowlen) {
+                                         int4* __restrict__ tface, int4* __restrict__ tmult, const Own& own) {
   const int s0 = (int)(4 * t);
   int out[4];
 #pragma unroll
@@ -300,26 +290,14 @@ __device__ __forceinline__ void emit_tet(int64_t t, int4 v, int4 m, int fb, cons
     if (first_occurrence(mk, s0 + k)) {
       const int F = fb + first_rank(m, s0, k);
       out[k] = F;
-      face_tet[F] = make_int2((int)t, mk >= 0 ? (mk >> 2) : -1);
-      const int3 lf = local_face(v, k);
-      face_vtx[3 * (int64_t)F] = lf.x;
-      face_vtx[3 * (int64_t)F + 1] = lf.y;
-      face_vtx[3 * (int64_t)F + 2] = lf.z;
-      const int kind = mk >= 0 ? 0 : (mk == -1 ? 1 : 2);
-      face_kind[F] = (int8_t)kind;
-      if (flag) flag[F] = kind != 2;      // Neumann faces present: multipliers by a scan of the flags
-      if (mult_iota) {                    // none: l(F) = F
-        mult_iota[F] = F;
-        rowlen[F] = mk >= 0 ? 7 : 4;
-        if (F + 1 == nF) rowlen[F + 1] = 0;  // the scan reads one entry past the last row
-      }
+      own(F, mk >= 0 ? (mk >> 2) : -1, local_face(v, k), mk >= 0 ? 0 : (mk == -1 ? 1 : 2));
     } else {
       const int t2 = mk >> 2, k2 = mk & 3;
       out[k] = (int)((unsigned)(ofb[k] + first_rank(om[k], 4 * t2, k2)) | 0x80000000u);
     }
   }
   tface[t] = make_int4(out[0], out[1], out[2], out[3]);
-  if (mult_iota) {
+  if (tmult) {
     int o[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) o[k] = (int)((unsigned)(out[k] & PH_ID_MASK) | (comp(m, k) < 0 ? PH_BND_BIT : 0u));
@@ -341,44 +319,83 @@ __device__ __forceinline__ void load_owners(int64_t t, int4 m, const int4* __res
   }
 }
 
-// 5. per tet: face ids, T+/T-, T+'s tuple, kind and non-Neumann flag of the
+// 5. per tet: face ids, and T+/T-, T+'s tuple, kind and non-Neumann flag of the
 //    faces it owns (first occurrences).  Without Neumann faces (mult_iota
 //    given) every face has a multiplier, l(F) = F, so the tet also writes its
 //    slots' multiplier ids and, for the faces it owns, the row length 1 + 3
 //    per tet of the face (7 interior, 4 boundary); k_tet_mult is not needed.
-//    Each thread takes two tets, t and t + half, and issues all their loads
-//    before using any (its warps mostly wait on loads).
-__device__ __forceinline__ void face_emit_item(int64_t t0, const int4* __restrict__ tet, int64_t nE, const int4* __restrict__ mate4,
-                            const int32_t* __restrict__ fbase, int4* __restrict__ tface, int2* __restrict__ face_tet,
-                            int32_t* __restrict__ face_vtx, int8_t* __restrict__ face_kind,
-                            int32_t* __restrict__ flag, int32_t* __restrict__ mult_iota, int4* __restrict__ tmult,
-                            int32_t* __restrict__ rowlen, const unsigned* status) {
-  const int64_t half = (nE + 1) >> 1;
-  if (t0 >= half || failed(status)) return;
-  const int64_t t1 = t0 + half;
-  const bool has1 = t1 < nE;
+//    The faces owned by a block's tets are consecutive: they are staged in
+//    shared memory and written in runs.  (Written by their tets, in up to 28
+//    partly filled stores per warp, they bound the kernel by L1: 0.66 ms at
+//    17.9M tets, now 0.47.)
+constexpr int kEmitThreads = 256;
+
+__global__ void __launch_bounds__(kEmitThreads) k_face_emit(
+    const int4* __restrict__ tet, int64_t nE, const int4* __restrict__ mate4, const int32_t* __restrict__ fbase,
+    int4* __restrict__ tface, int2* __restrict__ face_tet, int32_t* __restrict__ face_vtx,
+    int8_t* __restrict__ face_kind, int32_t* __restrict__ flag, int32_t* __restrict__ mult_iota,
+    int4* __restrict__ tmult, int32_t* __restrict__ rowlen, const unsigned* status) {
+  __shared__ int2 s_tet[4 * kEmitThreads];
+  __shared__ int32_t s_vtx[12 * kEmitThreads];
+  __shared__ int8_t s_kind[4 * kEmitThreads];
+  if (failed(status)) return;
+  const int64_t first = blockIdx.x * (int64_t)kEmitThreads, t = first + threadIdx.x;
+  const int base = fbase[first], count = fbase[min(first + kEmitThreads, nE)] - base;
+  if (t < nE) {
+    const int4 v = tet[t], m = mate4[t];
+    const int fb = fbase[t];
+    int4 om[4];
+    int ofb[4];
+    load_owners(t, m, mate4, fbase, om, ofb);
+    emit_tet(t, v, m, fb, om, ofb, tface, mult_iota ? tmult : nullptr, [&](int F, int minus, int3 lf, int kind) {
+      const int i = F - base;
+      s_tet[i] = make_int2((int)t, minus);
+      s_vtx[3 * i] = lf.x;
+      s_vtx[3 * i + 1] = lf.y;
+      s_vtx[3 * i + 2] = lf.z;
+      s_kind[i] = (int8_t)kind;
+    });
+  }
+  __syncthreads();
   const int nF = fbase[nE];
-  const int4 v0 = tet[t0], m0 = mate4[t0];
-  const int fb0 = fbase[t0];
-  const int4 v1 = has1 ? tet[t1] : make_int4(0, 0, 0, 0);
-  const int4 m1 = has1 ? mate4[t1] : make_int4(-1, -1, -1, -1);
-  const int fb1 = has1 ? fbase[t1] : 0;
-  int4 om0[4], om1[4];
-  int ofb0[4], ofb1[4];
-  load_owners(t0, m0, mate4, fbase, om0, ofb0);
-  if (has1) load_owners(t1, m1, mate4, fbase, om1, ofb1);
-  emit_tet(t0, v0, m0, fb0, om0, ofb0, nF, tface, face_tet, face_vtx, face_kind, flag, mult_iota, tmult, rowlen);
-  if (has1)
-    emit_tet(t1, v1, m1, fb1, om1, ofb1, nF, tface, face_tet, face_vtx, face_kind, flag, mult_iota, tmult, rowlen);
+  for (int i = threadIdx.x; i < count; i += kEmitThreads) {
+    const int F = base + i, kind = s_kind[i];
+    face_tet[F] = s_tet[i];
+    face_kind[F] = (int8_t)kind;
+    if (flag) flag[F] = kind != 2;  // Neumann faces present: multipliers by a scan of the flags
+    if (mult_iota) {                // none: l(F) = F
+      mult_iota[F] = F;
+      rowlen[F] = kind == 0 ? 7 : 4;
+      if (F + 1 == nF) rowlen[F + 1] = 0;  // the scan reads one entry past the last row
+    }
+  }
+  for (int i = threadIdx.x; i < 3 * count; i += kEmitThreads) face_vtx[3 * (int64_t)base + i] = s_vtx[i];
 }
 
-__global__ void k_face_emit(const int4* __restrict__ tet, int64_t nE, const int4* __restrict__ mate4,
-                            const int32_t* __restrict__ fbase, int4* __restrict__ tface, int2* __restrict__ face_tet,
-                            int32_t* __restrict__ face_vtx, int8_t* __restrict__ face_kind,
-                            int32_t* __restrict__ flag, int32_t* __restrict__ mult_iota, int4* __restrict__ tmult,
-                            int32_t* __restrict__ rowlen, const unsigned* status) {
-  face_emit_item(blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
-      tet, nE, mate4, fbase, tface, face_tet, face_vtx, face_kind, flag, mult_iota, tmult, rowlen, status);
+// The same for one tet, its faces written directly.
+__device__ __forceinline__ void face_emit_item(int64_t t, const int4* tet, int64_t nE, const int4* mate4,
+                                               const int32_t* fbase, int4* tface, int2* face_tet, int32_t* face_vtx,
+                                               int8_t* face_kind, int32_t* flag, int32_t* mult_iota, int4* tmult,
+                                               int32_t* rowlen, const unsigned* status) {
+  if (failed(status)) return;
+  const int nF = fbase[nE];
+  const int4 m = mate4[t];
+  int4 om[4];
+  int ofb[4];
+  load_owners(t, m, mate4, fbase, om, ofb);
+  emit_tet(t, tet[t], m, fbase[t], om, ofb, tface, mult_iota ? tmult : nullptr, [&](int F, int minus, int3 lf, int kind) {
+    face_tet[F] = make_int2((int)t, minus);
+    face_vtx[3 * F] = lf.x;
+    face_vtx[3 * F + 1] = lf.y;
+    face_vtx[3 * F + 2] = lf.z;
+    face_kind[F] = (int8_t)kind;
+    if (flag) flag[F] = kind != 2;
+    if (mult_iota) {
+      mult_iota[F] = F;
+      rowlen[F] = kind == 0 ? 7 : 4;
+      if (F + 1 == nF) rowlen[F + 1] = 0;
+    }
+  });
 }
 
 // face area 1/2 |(P_z - P_x) x (P_y - P_x)| of the vertices p[0..2] = P_x, P_y,
@@ -686,7 +703,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_connect(const SmallMesh
   const int nF = small_scan(nE + 1, [&](int64_t i) { return i < nE ? ph::first_occurrences(mate4[i], (int)(4 * i)) : 0; },
                             m.newc);
   if (tid == 0) m.d_tot[0] = nF;
-  for (int64_t i = tid; i < (nE + 1) / 2; i += kSmallThreads)
+  for (int64_t i = tid; i < nE; i += kSmallThreads)
     face_emit_item(i, m.tet, nE, mate4, m.newc, m.tface, m.face_tet, m.face_vtx, m.face_kind, nN > 0 ? m.flag : nullptr,
                    nN > 0 ? nullptr : m.face_mult, m.tmult, m.rowlen, m.status);
   __syncthreads();
@@ -716,7 +733,7 @@ __global__ void __launch_bounds__(128) k_small_geom(const SmallMesh m) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (failed(m.status)) return;
   if (i < m.nE) {
-    tet_geom(m.coord, m.tet[i], i, m.nE >= kFixedMin, m.geo, m.gexp, m.vol, m.status);
+    tet_geom(m.coord, m.tet[i], i, m.nE >= ph::kFixedMin, m.geo, m.gexp, m.vol, m.status);
     return;
   }
   i -= m.nE;
@@ -994,7 +1011,7 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
                         reinterpret_cast<const int4*>(mate), nE));  // nF -> d_tot[0]
   if (nE > 0) {
     KernelTimer kt("k_face_emit", s, 2);
-    k_face_emit<<<grid_for((nE + 1) / 2), kThreads, 0, s>>>(
+    k_face_emit<<<grid_for(nE, kEmitThreads), kEmitThreads, 0, s>>>(
         m->tet, nE, reinterpret_cast<int4*>(mate), newc, m->tface, m->face_tet, m->face_vtx, m->face_kind, flag,
         nN > 0 ? nullptr : m->face_mult, m->tmult, rowlen, m->status);
     PH_CU(launched(), "k_face_emit");
