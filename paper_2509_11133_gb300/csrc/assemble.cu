@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(128) k_recover(int64_t nE, const double* __res
 }
 
 // Recovery from the element factor Qf/9 stored by ph_assemble.
-template <bool GN>
+template <bool GN, bool FIXED>
 __global__ void __launch_bounds__(128) k_recover_factored(int64_t nE, const double2* __restrict__ vol,
                                                           const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                           const double* __restrict__ face_area,
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(128) k_recover_factored(int64_t nE, const doub
                                                           const double* __restrict__ lambda, double* __restrict__ u) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
-  recover_element_factored<GN>(t, vol, tface, tmult, face_area, factor, six_over_c, f_face, gN, lambda, u);
+  recover_element_factored<GN, FIXED>(t, vol, tface, tmult, face_area, factor, six_over_c, f_face, gN, lambda, u);
 }
 
 bool finite_pos(double x) { return x > 0.0 && x < INFINITY; }
@@ -231,12 +231,11 @@ extern "C" ph_status ph_recover_factored(const ph_mesh* m, const double* factor,
   const double six_over_c = 6.0 / c;
   const unsigned grid = grid_for(m->nE, 128);
   KernelTimer kt("k_recover_factored", s);
-  if (gN_face != nullptr && m->nFn > 0)
-    k_recover_factored<true><<<grid, 128, 0, s>>>(m->nE, m->vol, m->tface, m->tmult, m->face_area, factor,
-                                                  six_over_c, f_face, gN_face, lambda, u);
-  else
-    k_recover_factored<false><<<grid, 128, 0, s>>>(m->nE, m->vol, m->tface, m->tmult, m->face_area, factor,
-                                                   six_over_c, f_face, gN_face, lambda, u);
+  const bool gn = gN_face != nullptr && m->nFn > 0, fixed = m->nE >= kFixedMin;
+  const auto kernel = gn ? (fixed ? k_recover_factored<true, true> : k_recover_factored<true, false>)
+                         : (fixed ? k_recover_factored<false, true> : k_recover_factored<false, false>);
+  kernel<<<grid, 128, 0, s>>>(m->nE, m->vol, m->tface, m->tmult, m->face_area, factor, six_over_c, f_face, gN_face,
+                              lambda, u);
   const cudaError_t e = launched();
   kt.stop();
   return cuda_status(e, "k_recover_factored");

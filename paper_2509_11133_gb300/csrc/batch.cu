@@ -90,13 +90,23 @@ __global__ void k_batch_recover(const ProbDesc* __restrict__ probs, const Tile* 
     const Tile tl = tiles[k];
     const ProbDesc& d = probs[tl.prob];
     if (!d.u) continue;
+    const bool fixed = d.nE >= ph::kFixedMin;
     for (int i = threadIdx.x; i < tl.count; i += blockDim.x) {
-      if (d.flags & 2)
-        recover_element_factored<true>(tl.start + i, d.vol, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f,
-                                       d.gN, d.lambda, d.u);
-      else
-        recover_element_factored<false>(tl.start + i, d.vol, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f,
-                                        d.gN, d.lambda, d.u);
+      const int64_t t = tl.start + i;
+      if (d.flags & 2) {
+        if (fixed)
+          recover_element_factored<true, true>(t, d.vol, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f, d.gN,
+                                               d.lambda, d.u);
+        else
+          recover_element_factored<true, false>(t, d.vol, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f, d.gN,
+                                                d.lambda, d.u);
+      } else if (fixed) {
+        recover_element_factored<false, true>(t, d.vol, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f, d.gN,
+                                              d.lambda, d.u);
+      } else {
+        recover_element_factored<false, false>(t, d.vol, d.tface, d.tmult, d.area, d.factor, d.six_over_c, d.f, d.gN,
+                                               d.lambda, d.u);
+      }
     }
   }
 }

@@ -239,4 +239,28 @@ FX_HD bool face_kernel(const int64_t g[6], int kg, double a, double c20, double 
   return true;
 }
 
+// ---------------------------------------------------------------------------
+// e = Q z for the packed upper triangle Q of a 4x4 matrix: both on the scale of
+// their largest entry, each row's four products summed in integers and rounded
+// once: a row's error is at most 2^-53.9 max|Q| max|z| before that (2^-56.5 in
+// the mean), where the fp64 chain may lose 4 x 2^-53.  False (fp64 takes it) for exponents out of range, zero Q
+// or z among them.
+// ---------------------------------------------------------------------------
+FX_HD bool product4(const double Q[10], const double z[4], double e[4]) {
+  int kq = -1023, kz = -1023;
+  for (int i = 0; i < 10; ++i) kq = kq > exponent(Q[i]) ? kq : exponent(Q[i]);
+  for (int m = 0; m < 4; ++m) kz = kz > exponent(z[m]) ? kz : exponent(z[m]);
+  if (kq < -400 || kq > 400 || kz < -400 || kz > 400) return false;
+  Half q[10], w[4];
+  for (int i = 0; i < 10; ++i) q[i] = split(from_double(Q[i], kq + 1));  // below 2^60: four products fit
+  for (int m = 0; m < 4; ++m) w[m] = split(from_double(z[m], kz + 1));
+  const int at[4][4] = {{0, 1, 2, 3}, {1, 4, 5, 6}, {2, 5, 7, 8}, {3, 6, 8, 9}};
+  for (int k = 0; k < 4; ++k) {
+    Acc a(4);
+    for (int m = 0; m < 4; ++m) mac(a, q[at[k][m]], w[m]);
+    e[k] = to_double(shifted(a, 4), kq + kz - 58);
+  }
+  return true;
+}
+
 }  // namespace fx

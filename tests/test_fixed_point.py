@@ -26,6 +26,7 @@ extern "C" int run(const double* e, double a, double c20, double rdet, double* Q
   if (!fx::geometry(E, g, kg)) return 0;
   return fx::face_kernel(g, kg, a, c20, rdet, [](double x) { return 1.0 / x; }, Q) ? 2 : 1;
 }
+extern "C" int product(const double* Q, const double* z, double* e) { return fx::product4(Q, z, e); }
 extern "C" double there_and_back(double x, int k) { return fx::to_double(fx::from_double(x, k), k - 60); }
 """
 
@@ -41,6 +42,7 @@ def lib(tmp_path_factory):
     L = ctypes.CDLL(str(so))
     D = ctypes.c_double
     L.run.argtypes = [ctypes.POINTER(D), D, D, D, ctypes.POINTER(D)]
+    L.product.argtypes = [ctypes.POINTER(D)] * 3
     L.there_and_back.argtypes, L.there_and_back.restype = [D, ctypes.c_int], D
     return L
 
@@ -108,6 +110,29 @@ def test_against_rationals(lib, kind):
             big = max(abs(x) for x in ref)
             assert max(abs(Fraction(float(q)) - x) for q, x in zip(Q, ref)) <= Fraction(8 * 2.0 ** -53) * big
     assert taken >= 60
+
+
+@pytest.mark.parametrize("spread", [0, 3, 30])
+def test_product(lib, spread):
+    """Rows of Q z over `spread` decades of entries: 2^-53.9 of max|Q| max|z|, then rounded."""
+    rng = np.random.default_rng(spread)
+    P = ctypes.POINTER(ctypes.c_double)
+    at = [[0, 1, 2, 3], [1, 4, 5, 6], [2, 5, 7, 8], [3, 6, 8, 9]]
+    for i in range(300):
+        Q = rng.uniform(-2, 2, 10) * 10.0 ** rng.uniform(-spread, 0, 10) * 10.0 ** rng.uniform(-30, 30)
+        z = rng.uniform(-2, 2, 4) * 10.0 ** rng.uniform(-spread, 0, 4) * 10.0 ** rng.uniform(-30, 30)
+        if i % 5 == 0:
+            Q[i % 10], z[i % 4] = 0.0, np.nextafter(2.0, 0) * 2.0 ** 3
+        e = np.zeros(4)
+        assert lib.product(Q.ctypes.data_as(P), z.ctypes.data_as(P), e.ctypes.data_as(P)) == 1
+        scale = Fraction(float(np.abs(Q).max())) * Fraction(float(np.abs(z).max()))
+        for k in range(4):
+            ref = sum(Fraction(float(Q[at[k][m]])) * Fraction(float(z[m])) for m in range(4))
+            assert abs(Fraction(float(e[k])) - ref) <= Fraction(2.0 ** -53.9) * scale + Fraction(2.0 ** -53) * abs(ref)
+    for bad in (np.nan, np.inf):
+        Q[3] = bad
+        assert lib.product(Q.ctypes.data_as(P), z.ctypes.data_as(P), e.ctypes.data_as(P)) == 0
+    assert lib.product(np.zeros(10).ctypes.data_as(P), z.ctypes.data_as(P), e.ctypes.data_as(P)) == 0
 
 
 def test_left_to_fp64(lib):
