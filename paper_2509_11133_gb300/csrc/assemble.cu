@@ -38,7 +38,7 @@ using namespace ph_elem;
 
 namespace {
 
-// Fixed-point kernel: 58 FP64 operations per element where fp64 took 114 (17.9M
+// Fixed-point kernel: 60 FP64 operations per element where fp64 took 114 (17.9M
 // tets: 3.70 -> 2.31 ms; the FP64 pipe alone needs 1.9).  Six blocks of 128
 // threads per SM (80 registers): 4 (122 registers), 5 and 7 take 2.70, 2.40
 // and 2.31 ms.

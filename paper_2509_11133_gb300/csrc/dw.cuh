@@ -8,9 +8,7 @@
 // Popescu, "Tight and rigorous error bounds for basic building blocks of
 // double-word arithmetic", ACM TOMS 44(2), 2017 (u = 2^-24):
 //   add(DW, DW)  their AccurateDWPlusDW,  relative error <= 3u^2 + 13u^3
-//   add(DW, FP)  DWPlusFP,                <= 2u^2
 //   mul(DW, DW)  DWTimesDW3 (with fma),   <= 4u^2
-//   mul(DW, FP)  DWTimesFP3,              <= 2u^2
 // so a double-word value carries ~48 bits, against fp64's 53.  Every float
 // operation below is an explicit round-to-nearest intrinsic, so the compiler
 // cannot contract or reorder what the transforms rely on.
@@ -51,14 +49,6 @@ __device__ __forceinline__ f2 add(f2 x, f2 y) {
   return fast_two_sum(v.h, __fadd_rn(t.l, v.l));
 }
 
-__device__ __forceinline__ f2 add(f2 x, float y) {
-  const f2 s = two_sum(x.h, y);
-  return fast_two_sum(s.h, __fadd_rn(x.l, s.l));
-}
-
-__device__ __forceinline__ f2 neg(f2 x) { return {-x.h, -x.l}; }
-__device__ __forceinline__ f2 sub(f2 x, f2 y) { return add(x, neg(y)); }
-
 __device__ __forceinline__ f2 mul(f2 x, f2 y) {
   const float ch = __fmul_rn(x.h, y.h);
   const float cl1 = __fmaf_rn(x.h, y.h, -ch);
@@ -67,31 +57,8 @@ __device__ __forceinline__ f2 mul(f2 x, f2 y) {
   return fast_two_sum(ch, __fadd_rn(cl1, cl2));
 }
 
-__device__ __forceinline__ f2 mul(f2 x, float y) {
-  const float ch = __fmul_rn(x.h, y);
-  const float cl1 = __fmaf_rn(x.h, y, -ch);
-  return fast_two_sum(ch, __fmaf_rn(x.l, y, cl1));
-}
-
 // x * y + z
 __device__ __forceinline__ f2 fma(f2 x, f2 y, f2 z) { return add(mul(x, y), z); }
-
-// 1/y: the float reciprocal t, then one Newton step in double-word,
-// t + t (1 - y t); relative error ~ (2^-23)^2 + a few u^2.  y normal, nonzero.
-__device__ __forceinline__ f2 rcp(f2 y) {
-  const float t = __frcp_rn(y.h);
-  const f2 e = add(neg(mul(y, t)), 1.0f);  // 1 - y t, small
-  return add(mul(e, t), t);
-}
-
-// Binade of a nonzero normal float (bit pattern).
-__device__ __forceinline__ int exponent(float x) { return (int)((__float_as_uint(x) >> 23) & 0xFF) - 127; }
-
-// x * 2^p for an integer p in [-126, 127] (exact while the result is normal)
-__device__ __forceinline__ f2 ldexp(f2 x, int p) {
-  const float s = __uint_as_float((unsigned)(p + 127) << 23);
-  return {__fmul_rn(x.h, s), __fmul_rn(x.l, s)};
-}
 
 // Unbiased binary exponent of a finite nonzero double (bit pattern).
 __device__ __forceinline__ int exponent(double x) { return (int)((__double2hiint(x) >> 20) & 0x7FF) - 1023; }

@@ -242,9 +242,10 @@ FX_HD bool face_kernel(const int64_t g[6], int kg, double a, double c20, double 
 // ---------------------------------------------------------------------------
 // e = Q z for the packed upper triangle Q of a 4x4 matrix: both on the scale of
 // their largest entry, each row's four products summed in integers and rounded
-// once: a row's error is at most 2^-53.9 max|Q| max|z| before that (2^-56.5 in
-// the mean), where the fp64 chain may lose 4 x 2^-53.  False (fp64 takes it) for exponents out of range, zero Q
-// or z among them.
+// once.  Before that a row's error is at most 6 x 2^-56 max|Q| max|z| (the low
+// products, and the bits cut from the smaller entries; 2^-56.5 in the mean),
+// where the fp64 chain may lose 10 x 2^-53.  False (fp64 takes it) for exponents
+// out of range, zero Q or z among them.
 // ---------------------------------------------------------------------------
 FX_HD bool product4(const double Q[10], const double z[4], double e[4]) {
   int kq = -1023, kz = -1023;
