@@ -59,10 +59,11 @@ HBM_PEAK_FALLBACK = 6800.0
 FP64_PEAK_DERIVED_GOPS = 152 * 2 * 2.070
 # DFMA iterations per thread of one ph_fp64_peak launch (tens of ms)
 FP64_PEAK_ITERS = 4000
-# FP64 operations per element in k_assemble's formulas (each fma, add, mul or
-# div counted once): condensation kernel Qf 56, load and right-hand side 30,
-# condensed entries 24 (d_k (Q_km d_m + e_m) for the 10 entries, e_m = d_m/(c|T|)).
-ASSEMBLE_OPS_PER_TET = 110
+# FP64 operations per element in k_assemble (each fma, add, mul or div counted
+# once): load and right-hand side 30, condensed entries 24 (d_k (Q_km d_m + e_m)
+# for the 10 entries, e_m = d_m/(c|T|)), reciprocal and scale of the condensation
+# kernel Qf 6; its products are integers.
+ASSEMBLE_OPS_PER_TET = 60
 # Method-level bytes per element of the numeric phase: coordinates, f and
 # H counted once (136 + 24 nC/nE + 24 nF/nE).
 def assemble_bytes_per_tet(nE, nC, nF):
@@ -553,13 +554,11 @@ def variant_report(v, nE, nC, nF, world, fp64_peak_gops, hbm_peak, f64_step_ms, 
     prof = profile_figures("k_assemble_dw")
     bpt = assemble_bytes_per_tet(nE, nC, nF)
     out = {
-        "what": "ph_mesh_create_dw + ph_assemble_dw + ph_recover_factored_dw: the element geometry (G_e, "
-                "G_e T0^-1), the condensation kernel (the 3x3 algebra of A^-1) and the recovery's product "
-                "(Qf/9) z' in double-word arithmetic (float pairs, ~48 bits) on the FP32 pipe; edge vectors, "
-                "|det E|, face areas, the leading term d d'/(c|T|), every sum of H and rhs and the recovery's "
-                "z' terms in fp64; flat or reaction-dominated elements take the fp64 kernel; tested against the "
-                "oracle at the fp64 path's bars",
-        "dtype": "f64 + f32x2 (double-word) geometry and condensation kernel",
+        "what": "ph_mesh_create_dw + ph_assemble_dw + ph_recover_factored_dw: the mesh build and the condensation "
+                "of the fp64 path (products in 64-bit fixed point), the recovery's product (Qf/9) z' in "
+                "double-word arithmetic (float pairs, ~48 bits) on the FP32 pipe; tested against the oracle at "
+                "the fp64 path's bars",
+        "dtype": "f64 + f32x2 (double-word) recovery product",
         "value": whole_job_rate(nE, world, v["step_ms"]), "unit": UNIT, "ms_per_step": v["step_ms"],
         "phases_ms": v["phases_ms"], "mesh_build_kernels_ms": v["mesh_build_kernels_ms"],
         "speedup_step_vs_f64": f64_step_ms / v["step_ms"],

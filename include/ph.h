@@ -290,8 +290,9 @@ ph_status ph_solve_pcg_noalloc(int64_t n, const int32_t* rowptr, const int32_t* 
 /*
  * Batched assembly (not in the paper): many problems, meshes of uneven size
  * each with its own coefficient field, assembled and condensed by one
- * persistent kernel (plus one kernel that clears values and rhs first).  Each problem's values, rhs and factor are bit-identical to
- * a plain ph_assemble call on it.  A batch is not thread-safe.
+ * persistent kernel (plus one kernel that clears values and rhs first).  Each
+ * problem's values, rhs and factor are bit-identical to a plain ph_assemble
+ * call on it.  A batch is not thread-safe.
  *   ph_batch_create   group n meshes (the meshes must outlive the batch).
  *   ph_batch_bind     per-problem arrays: host arrays of n DEVICE pointers
  *                     (uD_face, gN_face, factor may be NULL arrays or hold

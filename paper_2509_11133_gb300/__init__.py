@@ -266,7 +266,7 @@ class Mesh:
 
     ``coord`` (nC x 3 float64) and ``tet`` (nE x 4 int32) are CUDA tensors;
     ``neumann`` (nN x 3 int32) optional.  geometry "dw" builds with
-    ph_mesh_create_dw (double-word geometry record, for ph_assemble_dw).
+    ph_mesh_create_dw (a mesh for ph_assemble_dw).
     Methods allocate outputs with torch and call the matching ``ph_*`` entry
     point on the current stream.
     """
@@ -350,7 +350,7 @@ class Mesh:
                  variant="f64"):
         """H values and rhs; with ``factor`` (nE*10 float64, or True to
         allocate) also the element factor for recover_factored.  variant
-        "dw" runs ph_assemble_dw (condensation kernel in double-word)."""
+        "dw" runs ph_assemble_dw."""
         _need(a, torch.float64, self.nE, "a")
         _need(f_face, torch.float64, self.nF, "f_face")
         if uD_face is not None:
