@@ -137,10 +137,11 @@ __global__ void k_face_count(const int4* __restrict__ tet, int64_t nE, int64_t n
 //    same thread then computes the tet's geometry: G_e in fixed point on the
 //    integer pipe (fixed.cuh), 22 FP64 operations where the fp64 record took
 //    55 and bound the kernel.  Now the atomics, the scattered stores and the
-//    geometry share it (17.9M tets: 1.94 -> 1.09 ms).  Blocks of 128 threads, 6
-//    per SM (80 registers): 5 or 7 take 1.15 and 1.09 ms, 256-thread blocks
-//    at 96 registers 1.63; storing the entries after the geometry instead of
-//    before it holds their stores back, 1.26.
+//    geometry share it (17.9M tets: 1.94 -> 1.10 ms; 1.08 without the low
+//    products, which cost graded elements accuracy).  Blocks of 128 threads, 6
+//    per SM (80 registers): without those, 5 or 7 took 1.15 and 1.09 ms,
+//    256-thread blocks at 96 registers 1.63; storing the entries after the
+//    geometry instead of before it holds their stores back, 1.26.
 constexpr int kFillThreads = 128;
 template <bool GEO>
 __device__ __forceinline__ void face_fill_item(int64_t i, const int4* __restrict__ tet, int64_t nE, int64_t nC, const int32_t* __restrict__ nb,
