@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(128) k_recover(int64_t nE, const double* __res
   const double2 vt = __ldg(vol + t);
   const Record R = load_record(geo, gexp, t);
   double z[4];
-  recovery_load<GN>(vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
+  recovery_load(GN, vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
   double Q[10];
   element_kernel(R, vt, at, c20, Q);  // Qf/9
   const double icT = vt.y * six_over_c;
@@ -94,9 +94,11 @@ __global__ void __launch_bounds__(128) k_recover(int64_t nE, const double* __res
   store_u(u, t, U);
 }
 
-// Recovery from the element factor Qf/9 stored by ph_assemble.
+// Recovery from the element factor Qf/9 stored by ph_assemble.  FIXED: seven
+// blocks per SM (72 registers, 24 bytes of spills; unbounded 84); 17.9M tets 0.745
+// ms, 5 and 8 blocks 0.84 and 0.75.
 template <bool GN, bool FIXED>
-__global__ void __launch_bounds__(128) k_recover_factored(int64_t nE, const double2* __restrict__ vol,
+__global__ void __launch_bounds__(128, FIXED ? 7 : 8) k_recover_factored(int64_t nE, const double2* __restrict__ vol,
                                                           const int4* __restrict__ tface, const int4* __restrict__ tmult,
                                                           const double* __restrict__ face_area,
                                                           const double* __restrict__ factor, double six_over_c,
@@ -105,7 +107,7 @@ __global__ void __launch_bounds__(128) k_recover_factored(int64_t nE, const doub
                                                           const double* __restrict__ lambda, double* __restrict__ u) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nE) return;
-  recover_element_factored<GN, FIXED>(t, vol, tface, tmult, face_area, factor, six_over_c, f_face, gN, lambda, u);
+  recover_element_factored(GN, FIXED, t, vol, tface, tmult, face_area, factor, six_over_c, f_face, gN, lambda, u);
 }
 
 bool finite_pos(double x) { return x > 0.0 && x < INFINITY; }

@@ -238,8 +238,7 @@ __device__ __forceinline__ void store_u(double* __restrict__ u, int64_t t, const
 }
 
 // z'_k = |T|/4 f(Ct_k) + |F_k| g(Ct_k) [Neumann] + d_k Lambda_k
-template <bool GN>
-__device__ __forceinline__ void recovery_load(double q4, int4 tf, int4 tm, const double* __restrict__ face_area,
+__device__ __forceinline__ void recovery_load(bool GN, double q4, int4 tf, int4 tm, const double* __restrict__ face_area,
                                               const double* __restrict__ f_face, const double* __restrict__ gN,
                                               const double* __restrict__ lambda, double z[4]) {
 #pragma unroll
@@ -261,9 +260,12 @@ __device__ __forceinline__ void recovery_load(double q4, int4 tf, int4 tm, const
 // (Algorithm 1, second loop): U[o(k)] = z'sum/(c|T|) - 3 (Qf/9 z')_k.  The
 // body of the plain and the batched recovery kernels.
 // FIXED: the product in fixed point (fixed.cuh), 18 FP64 operations instead of
-// 34, which bound the kernel (17.9M tets: 1.09 -> 0.70 ms).
-template <bool GN, bool FIXED>
-__device__ __forceinline__ void recover_element_factored(int64_t t, const double2* __restrict__ vol,
+// 34, which bound the kernel (17.9M tets: 1.09 -> 0.745 ms).  A row that it leaves
+// out (one in some hundreds of random fields) reads its factor again: held in
+// registers for that, the kernel took 0.96 ms.
+// (GN, FIXED: constants of the plain kernels, the problem's in the batched one.)
+__device__ __forceinline__ void recover_element_factored(bool GN, bool FIXED, int64_t t,
+                                                         const double2* __restrict__ vol,
                                                          const int4* __restrict__ tface,
                                                          const int4* __restrict__ tmult,
                                                          const double* __restrict__ face_area,
@@ -273,14 +275,26 @@ __device__ __forceinline__ void recover_element_factored(int64_t t, const double
                                                          const double* __restrict__ lambda, double* __restrict__ u) {
   const double2 vt = __ldg(vol + t);
   double z[4];
-  recovery_load<GN>(vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
+  recovery_load(GN, vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
   const double2* fp = reinterpret_cast<const double2*>(factor + 10 * t);
   const double2 q0 = __ldg(fp), q1 = __ldg(fp + 1), q2 = __ldg(fp + 2), q3 = __ldg(fp + 3), q4 = __ldg(fp + 4);
   const double Q[10] = {q0.x, q0.y, q1.x, q1.y, q2.x, q2.y, q3.x, q3.y, q4.x, q4.y};
   const double icT = vt.y * six_over_c;
   const double zs = icT * ((z[0] + z[1]) + (z[2] + z[3]));
   double e[4], U[4];
-  if (!FIXED || !fx::product4(Q, z, e)) {
+  if (FIXED) {
+    unsigned rows;  // to form in fp64, as the other branch does
+    if (!fx::product4(Q, z, e, &rows)) rows = 0xF;
+    while (rows) {
+      const int k = __ffs(rows) - 1;
+      rows &= rows - 1;
+      double s = 0.0;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) s = fma(__ldg(factor + 10 * t + ut(k, m)), z[m], s);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) e[j] = j == k ? s : e[j];
+    }
+  } else {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       e[k] = 0.0;
@@ -315,7 +329,7 @@ __device__ __forceinline__ void recover_element_factored_dw(int64_t t, const dou
   using namespace dw;
   const double2 vt = __ldg(vol + t);
   double z[4];
-  recovery_load<GN>(vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
+  recovery_load(GN, vt.x * (1.0 / 24.0), __ldg(tface + t), __ldg(tmult + t), face_area, f_face, gN, lambda, z);
   const double2* fp = reinterpret_cast<const double2*>(factor + 10 * t);
   const double2 q0 = __ldg(fp), q1 = __ldg(fp + 1), q2 = __ldg(fp + 2), q3 = __ldg(fp + 3), q4 = __ldg(fp + 4);
   const double Q[10] = {q0.x, q0.y, q1.x, q1.y, q2.x, q2.y, q3.x, q3.y, q4.x, q4.y};

@@ -1,6 +1,6 @@
 """The fixed-point element algebra (csrc/fixed.cuh, compiled here for the CPU)
 against exact rational arithmetic where entries of one element differ in size:
-edges and faces of a graded mesh."""
+edges and faces of a graded mesh, rows of Q z over several decades."""
 import ctypes
 import os
 import subprocess
@@ -18,6 +18,9 @@ extern "C" int gram(const double* e, double* G) {
   if (!fx::geometry(reinterpret_cast<const double(*)[3]>(e), g, kg)) return 0;
   for (int i = 0; i < 6; ++i) G[i] = fx::to_double(g[i], kg);
   return 1;
+}
+extern "C" int product(const double* Q, const double* z, double* e, unsigned* small) {
+  return fx::product4(Q, z, e, small);
 }
 """
 U = 2.0 ** -53
@@ -79,3 +82,35 @@ def test_gram_entries(lib, kind, inv):
             scale = float(ref[i, i] * ref[j, j]) ** 0.5
             assert abs(float(Fraction(float(G[n])) - ref[i, j])) <= 2.05 * U * scale
     assert taken >= 150 or inv > 4  # the rest are left to fp64
+
+
+@pytest.mark.parametrize("spread", [0, 1, 2, 4, 8])
+def test_product_rows(lib, spread):
+    """Each row of Q z that is not marked for fp64, to 8 x 2^-53 of its own terms:
+    one for the rounding to fp64, one for half a unit of the sum (2^-60 of
+    max|Q| max|z|, of which the row's largest term is at least 2^-7), and two
+    (a unit) for each of the three other terms if an operand of it is cut.  The
+    root mean square stays below fp64's own chain, and most rows are taken."""
+    rng = np.random.default_rng(spread)
+    at = [[0, 1, 2, 3], [1, 4, 5, 6], [2, 5, 7, 8], [3, 6, 8, 9]]
+    taken, err, err64 = 0, [], []
+    n = 500
+    for _ in range(n):
+        Q = rng.uniform(-2, 2, 10) * 10.0 ** rng.uniform(-spread, 0, 10)
+        z = rng.uniform(-2, 2, 4) * 10.0 ** rng.uniform(-spread, 0, 4)
+        e, small = np.zeros(4), ctypes.c_uint(0)
+        assert lib.product(ptr(Q), ptr(z), ptr(e), ctypes.byref(small)) == 1
+        for k in range(4):
+            if small.value >> k & 1:
+                continue
+            taken += 1
+            f = [Fraction(float(Q[at[k][m]])) * Fraction(float(z[m])) for m in range(4)]
+            terms = float(sum(abs(x) for x in f))
+            chain = 0.0
+            for x in f:  # the fma chain: each sum rounded once
+                chain = float(Fraction(chain) + x)
+            err.append(abs(float(Fraction(float(e[k])) - sum(f))) / terms)
+            err64.append(abs(float(Fraction(chain) - sum(f))) / terms)
+    assert max(err) <= 8 * U
+    assert np.mean(np.square(err)) <= np.mean(np.square(err64))
+    assert taken >= (4 * n if spread == 0 else n) * 0.9
