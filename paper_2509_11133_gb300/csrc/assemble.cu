@@ -39,8 +39,8 @@ using namespace ph_elem;
 namespace {
 
 // Fixed-point kernel: 60 FP64 operations per element where fp64 took 114 (17.9M
-// tets: 3.70 -> 2.34 ms; the FP64 pipe alone needs 1.9).  Six blocks of 128
-// threads per SM (80 registers; 8 to 16 bytes of spills in half of the
+// tets: 3.70 -> 2.37 ms; the FP64 pipe alone needs 1.9).  Six blocks of 128
+// threads per SM (80 registers; 4 to 16 bytes of spills in most of the
 // instances): 4 (122 registers), 5 and 7 took 2.70, 2.40 and 2.31 ms where 6
 // took 2.31.
 template <bool UD, bool GN, bool FAC>

@@ -6,14 +6,16 @@
 // (assemble.cu) are sums of products of numbers of similar size, so they are
 // formed here in 64-bit integers with one power of two per element: a product
 // of two such numbers takes three IMAD.WIDE (0.2 clocks, against 0.57 for a
-// DFMA) on a pipe that the FP64 kernels leave idle, and rounds at 2^-55 to
-// 2^-59 of the result's scale, below fp64's 2^-53.  The results return to
-// fp64 rounded to nearest.
+// DFMA) on a pipe that the FP64 kernels leave idle.  The results return to fp64
+// rounded to nearest.
 //
 // A number is an int64 v with |v| < 2^61 (up to 2^62 where noted) and a scale
 // known per element.  A product uses v = h 2^32 + l with l a signed 32-bit
 // integer: sum of v w = 2^64 sum(h h') + 2^32 sum(h l' + l h') + sum(l l'),
-// and the last sum, below 2^62 per term, is left out (mac_wide keeps it).
+// and the last sum, below 2^62 per term, is left out where the result keeps no bits
+// below it, and kept (mac_wide) where the sum is shifted further: left out of Y
+// (a shift of 6) it cost Q up to 10.7 x 2^-53 of its largest entry, now 4.2 at worst
+// and 1.4 rms at most over the shapes that are accepted; fp64: 17 and 3.4.
 // Sums of at most three products do not overflow with |v|, |w| <= 2^61:
 // |h l'| <= 2^60, six of them 2^62.6.  The high sum may be shifted past 2^63 on
 // the way (two's complement): only the final value has to fit.
@@ -214,10 +216,10 @@ FX_HD bool face_kernel(const int64_t g[6], int kg, double a, double c20, double 
   };
   const Half A00 = two(m11, m22, n12, m12), A01 = two(m02, m12, n01, m22), A02 = two(m01, m12, n02, m11);
   const Half A11 = two(m00, m22, n02, m02), A12 = two(m01, m02, n12, m00), A22 = two(m00, m11, n01, m01);
-  Acc d;
-  mac(d, m00, A00);
-  mac(d, m01, A01);
-  mac(d, m02, A02);
+  Acc d(6);
+  mac_wide(d, m00, A00);
+  mac_wide(d, m01, A01);
+  mac_wide(d, m02, A02);
   const int64_t D = shifted(d, 6);
   if (D <= 0) return false;
   const Half s = split(from_double((6.0 / 9.0 * rdet) * rcp(to_double(D, 0)), kr - 57));
@@ -229,10 +231,10 @@ FX_HD bool face_kernel(const int64_t g[6], int kg, double a, double c20, double 
   const Half t10 = split(g[1] - r1), t11 = split(g[3] - r1), t12 = split(g[4] - r1);
   const Half t20 = split(g[2] - r2), t21 = split(g[4] - r2), t22 = split(g[5] - r2);
   const auto three = [](Half p, Half q, Half r, Half t, Half u, Half v) {
-    Acc y;
-    mac(y, p, q);
-    mac(y, r, t);
-    mac(y, u, v);
+    Acc y(6);
+    mac_wide(y, p, q);
+    mac_wide(y, r, t);
+    mac_wide(y, u, v);
     return shifted(y, 6);
   };
   const int64_t y00 = three(B00, t00, B01, t10, B02, t20), y01 = three(B00, t01, B01, t11, B02, t21);

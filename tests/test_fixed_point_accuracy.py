@@ -9,6 +9,8 @@ from fractions import Fraction
 import numpy as np
 import pytest
 
+from tests.test_fixed_point import exact
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SRC = r"""
 #include "fixed.cuh"
@@ -18,6 +20,12 @@ extern "C" int gram(const double* e, double* G) {
   if (!fx::geometry(reinterpret_cast<const double(*)[3]>(e), g, kg)) return 0;
   for (int i = 0; i < 6; ++i) G[i] = fx::to_double(g[i], kg);
   return 1;
+}
+extern "C" int kernel(const double* e, double a, double c20, double rdet, double* Q) {
+  int64_t g[6];
+  int kg;
+  return fx::geometry(reinterpret_cast<const double(*)[3]>(e), g, kg) &&
+         fx::face_kernel(g, kg, a, c20, rdet, [](double x) { return 1.0 / x; }, Q);
 }
 extern "C" int product(const double* Q, const double* z, double* e, unsigned* small) {
   return fx::product4(Q, z, e, small);
@@ -82,6 +90,53 @@ def test_gram_entries(lib, kind, inv):
             scale = float(ref[i, i] * ref[j, j]) ** 0.5
             assert abs(float(Fraction(float(G[n])) - ref[i, j])) <= 2.05 * U * scale
     assert taken >= 150 or inv > 4  # the rest are left to fp64
+
+
+# e (three edges), a, c/20, 1/|det E|: elements whose Q was off by 9.3 to 10.7 x
+# 2^-53 of its largest entry without the low products of Y = adj(M) G T0^-1
+HARD = """
+0x1.9561ba82a07e7p-2 0x1.dae5897fb548p-5 0x1.c9ea7531d9978p-3 0x1.972cc0cfb6618p-4 0x1.8f8c2a2304d8ap-2 0x1.b6e17524bbdf8p-3 0x1.21d3571bec14p-3 0x1.0f883f9ae7818p-4 0x1.fba1cbb304d08p-2 0x1.cdf15f3789537p-2 0x1.a94e01d67dabfp-13 0x1.0f48cc2612c6ap+4
+0x1.9cc8aa31521ap-7 0x1.897ae9b8b18p-10 0x1.73f3c1fb74p-13 0x1.991b9c2b8e2cp-6 0x1.e589b4d28fd6p-6 0x1.8a540e77bf0bp-9 0x1.b092db12e15cp-6 0x1.cc52f8cf5915p-6 0x1.803bb4bfb7f9ap-6 0x1.d44ec52224243p+3 0x1.42cd70f8a22bp-7 0x1.1a67fdc4e4b79p+17
+0x1.2304dfef43cp-14 0x1.02528414414p-11 0x1.372e4ed29p-15 -0x1.8b8ebbc280bp-13 0x1.4cb8e87081p-9 0x1.868123ee093p-9 0x1.15ca3ec0372ap-10 0x1.98b27ddaf42p-9 0x1.277a4a81a27p-9 0x1.b434e1085a4edp-2 0x1.9257e876084p-9 0x1.5597024a8d2e3p+29
+0x1.0f2c915fd3418p-5 -0x1.0909b1505f61p-5 0x1.91a6e76812p-12 0x1.eb0a1da33048p-9 -0x1.f09dcc3da2dep-6 0x1.bbf798ad3b48p-9 0x1.26ba5814858cp-8 -0x1.2125055313edp-5 0x1.2f2029f088bdp-6 0x1.cee20a90a00bdp-4 0x1.49f261455c3c8p-6 0x1.2fdf960a4a796p+16
+0x1.5da048293224p-7 0x1.000daa255228p-8 -0x1.25762759958p-9 0x1.114646b2b0fp-7 0x1.61d66d1003dp-9 -0x1.27b72f33448p-12 0x1.44b7f2d595cp-8 0x1.18bd77e1dbfp-9 -0x1.bf75c0f214p-12 0x1.f468f18deee99p-3 0x1.a03d7881631a4p-8 0x1.00203304e30a7p+27
+-0x1.201252cf296ap-4 -0x1.02c8e6225254p-6 0x1.21ca8a0adbb1p-6 -0x1.fe0f695b1c7ap-5 -0x1.1aeaa0a41954ap-3 -0x1.c1b8fad895c4p-8 -0x1.ae79deb360b1p-5 -0x1.452601dc3ff36p-3 0x1.e179c2bea91dp-5 0x1.74422163603dp+0 0x1.05de68724f06fp-11 0x1.8c7368072b8acp+10
+"""
+
+
+@pytest.mark.parametrize("row", HARD.split("\n")[1:-1], ids=range(6))
+def test_condensation_of_hard_elements(lib, row):
+    """Q to 8 x 2^-53 of its largest entry: the scalar's fp64 operations (five:
+    the constant, two products, a reciprocal, det M's conversion), the rounding to
+    fp64, and less than one each for det M (2^-54.7) and for the sums."""
+    v = np.array([float.fromhex(x) for x in row.split()])
+    e, (a, c20, rdet) = np.ascontiguousarray(v[:9]), v[9:]
+    Q = np.zeros(10)
+    D = ctypes.c_double
+    assert lib.kernel(ptr(e), D(a), D(c20), D(rdet), ptr(Q)) == 1
+    ref = exact(e.reshape(3, 3), a, c20, rdet)
+    big = max(abs(x) for x in ref)
+    assert max(abs(Fraction(float(q)) - x) for q, x in zip(Q, ref)) <= Fraction(8 * U) * big
+
+
+def test_condensation_of_needles(lib):
+    """The same bound on elements that are nearly collinear or coplanar off the axes."""
+    rng = np.random.default_rng(2)
+    taken = 0
+    for i in range(200):
+        e = graded(("needle", "flat")[i % 2], float(rng.uniform(4, 40)), rng)
+        rdet = 1.0 / abs(np.linalg.det(e))
+        a = float(np.exp(rng.standard_normal()))
+        c20 = a / float((e ** 2).sum(1).max()) * 10.0 ** rng.uniform(-12, -1)
+        Q = np.zeros(10)
+        D = ctypes.c_double
+        if not lib.kernel(ptr(e), D(a), D(c20), D(rdet), ptr(Q)):
+            continue
+        taken += 1
+        ref = exact(e, a, c20, rdet)
+        big = max(abs(x) for x in ref)
+        assert max(abs(Fraction(float(q)) - x) for q, x in zip(Q, ref)) <= Fraction(8 * U) * big
+    assert taken >= 60
 
 
 @pytest.mark.parametrize("spread", [0, 1, 2, 4, 8])
