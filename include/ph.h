@@ -532,6 +532,9 @@ ph_status ph_kernel_time(const char* kernel, int reset, double* ms, int64_t* lau
  *     status word and return (every wait in the scan is bounded; nothing
  *     hangs).  Scans of fewer than three tiles (4096 values each) are not
  *     affected.  Off by default; for tests only.
+ *   ph_test_pcg_loop(mode): 1 makes the conjugate-gradient solves run their
+ *     per-iteration kernels where they would run all iterations in one launch
+ *     (the same bits); 0 (the default) does not.
  *   ph_pool_in_use(bytes): (host) bytes of the current device's library pool
  *     held by live allocations (freed memory counts once its stream-ordered
  *     free has run), to check that failed calls leak nothing.
@@ -540,6 +543,7 @@ ph_status ph_kernel_time(const char* kernel, int reset, double* ms, int64_t* lau
  */
 ph_status ph_test_fail_alloc(int64_t after);
 ph_status ph_test_scan_withhold(int on);
+ph_status ph_test_pcg_loop(int mode);
 ph_status ph_pool_in_use(int64_t* bytes);
 
 /*

@@ -36,7 +36,7 @@ EXPORTS = ("ph_mesh_create", "ph_mesh_destroy", "ph_mesh_info", "ph_mesh_faces",
            "ph_batch_graph_launch", "ph_refine", "ph_refined_info", "ph_refined_copy", "ph_refined_destroy", "ph_rcp", "ph_half_sqrt", "ph_timing_enable",
            "ph_kernel_time", "ph_assemble_host", "ph_schwarz_create", "ph_schwarz_destroy",
            "ph_solve_pcg_schwarz", "ph_fp64_peak", "ph_test_fail_alloc", "ph_test_scan_withhold",
-           "ph_pool_in_use", "ph_solve_refined", "ph_mesh_create_batch", "ph_host_mesh_query",
+           "ph_test_pcg_loop", "ph_pool_in_use", "ph_solve_refined", "ph_mesh_create_batch", "ph_host_mesh_query",
            "ph_assemble_dw", "ph_batch_bind_recovery", "ph_mesh_create_dw")
 
 
@@ -106,6 +106,7 @@ def load(path: str | None = None):
         "ph_fp64_peak": [I64, ctypes.POINTER(D), ctypes.POINTER(D), P],
         "ph_test_fail_alloc": [I64],
         "ph_test_scan_withhold": [ctypes.c_int],
+        "ph_test_pcg_loop": [ctypes.c_int],
         "ph_pool_in_use": [ctypes.POINTER(I64)],
         "ph_solve_refined": [P, P, P, P, P, D, D, I32, I32, ctypes.POINTER(I32), ctypes.POINTER(I32),
                              ctypes.POINTER(D), P],
@@ -536,6 +537,11 @@ def ph_test_fail_alloc(after):
 def ph_test_scan_withhold(on):
     """Test hook: scans withhold one tile's publication (bounded waits run out)."""
     _check(load().ph_test_scan_withhold(1 if on else 0), "ph_test_scan_withhold")
+
+
+def ph_test_pcg_loop(mode):
+    """Test hook: 1 keeps solves from the one-launch loop, 0 does not."""
+    _check(load().ph_test_pcg_loop(int(mode)), "ph_test_pcg_loop")
 
 
 def ph_pool_in_use() -> int:

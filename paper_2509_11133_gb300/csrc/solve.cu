@@ -313,19 +313,25 @@ inline cudaError_t pcg_iteration(int64_t n, const Matrix& A, double* x, double* 
 // grid, which for n <= kLoopMaxN means one row, or one pair of rows, per
 // thread), so the iterates, the iteration count and x are theirs bit for bit:
 // blocks publish the sums of single warps, or of virtual 256-thread blocks,
-// and every block finishes the same tree on them.  Per iteration, before and
-// after: 43 -> 10 us (Schwarz, 1,376 rows), 45 -> 14 us (Schwarz, 21,120),
-// 33 -> 10 us (Jacobi, 47,520); of 20,000 to 24,000 cycles, about 4,600 a
-// phase are the meeting (2,600), reading the sums (900, an L2 trip across the
-// dies), their tree and the division (69 cycles per dependent FP64 operation).
+// and every block finishes the same tree on them.  Us per iteration, the
+// kernels above and this loop, on jittered meshes:
+//     rows        1,650   9,234  21,600  50,688  98,400  169,344  297,714
+//     Jacobi     34  8   36 10   36 10   37 11   37 16    41 20    43 30
+//     Schwarz    47 12   47 14   47 15   47 17   51 24    57 33    64 41
+// so the loop takes every size that one row per thread allows.  Of a small
+// system's 20,000 to 24,000 cycles, about 4,600 a phase are the meeting (2,600),
+// reading the sums (900, an L2 trip across the dies), their tree and the division
+// (69 cycles per dependent FP64 operation).
 //
 // The meeting is a counter: each block adds one with release semantics after a
-// block barrier, and polls it.  (Polling tagged sums instead of a counter saves
-// the trip that then reads the sums, but 152 blocks polling 152 sums take
-// 7,100 cycles to see them all against 1,400.)  The vectors that other blocks
-// write are read by ld.cg, i.e. from L2, where the release has put them before
-// the count; nothing here acquires, since an acquire empties L1 of the matrix
-// and the patch inverses, which every phase reads again.
+// block barrier and polls it with acquire semantics before the next one, so that
+// what any thread wrote before a meeting happens before what any thread reads
+// after it.  (Polling tagged sums instead of a counter saves the trip that then
+// reads the sums, but 152 blocks polling 152 sums take 7,100 cycles to see them
+// all against 1,400.)  The acquire empties L1 of the matrix and the patch inverses,
+// which costs a 47,520-row Jacobi solve 6 to 12% and the Schwarz solves 2%; without
+// it nothing orders the reads.  A relaxed poll and an acquire at its end take the
+// same time, a relaxed poll and a fence 5 to 7% more.
 // ---------------------------------------------------------------------------
 struct LoopArgs {
   int64_t n;
@@ -348,8 +354,7 @@ struct LoopArgs {
 };
 
 // All blocks of the grid meet (they are co-resident: a cooperative launch).
-// Everything the block wrote before is in L2 when the others pass.  Bounded:
-// *late is set, and the call returns, when the wait runs out.
+// Bounded: *late is set, and the call returns, when the wait runs out.
 __device__ __forceinline__ void loop_meet(unsigned* bar, unsigned& target, int spin_limit, int* late) {
   __syncthreads();
   target += gridDim.x;
@@ -357,7 +362,7 @@ __device__ __forceinline__ void loop_meet(unsigned* bar, unsigned& target, int s
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     unsigned seen;
     for (int spins = 0;; ++spins) {
-      asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
       if ((int)(seen - target) >= 0) break;
       if (spins > spin_limit) {
         *late = 1;
@@ -738,6 +743,8 @@ __global__ void __launch_bounds__(RT, SCHW ? 2 : 3) k_pcg_loop(const __grid_cons
 }
 
 constexpr int kLoopSpinLimit = 1 << 21;  // polls (about a microsecond each)
+// Test hook (ph_test_pcg_loop): 1 keeps the solver from k_pcg_loop.
+std::atomic<int> g_test_pcg_loop{0};
 constexpr int kLoopIters = 4096;         // iterations per launch (a multiple of 16: the buffers end where they began)
 
 // Launch k_pcg_loop for the A.n rows: up to kLoopWarpN rows, one block per SM of
@@ -799,7 +806,8 @@ ph_status pcg_run(int64_t n, const int32_t* rowptr, const int32_t* colind, const
   void* ell = nullptr;
   // the whole iteration in one launch (k_pcg_loop) where n allows; with x not
   // 16-byte aligned the sums have another order, kept by the kernels above
-  bool loop = n <= kLoopMaxN && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+  const int hook = g_test_pcg_loop.load(std::memory_order_relaxed);
+  bool loop = n <= kLoopMaxN && (reinterpret_cast<uintptr_t>(x) & 15) == 0 && hook != 1;
   cudaError_t e = cudaMemsetAsync(sc, 0, sizeof(Scalars), s);
   if (e == cudaSuccess && ell_ok) {  // width of the longest row (read at the first synchronisation below)
     k_row_width<<<RB, RT, 0, s>>>(n, rowptr, &sc->done);
@@ -926,6 +934,12 @@ ph_status pcg_run(int64_t n, const int32_t* rowptr, const int32_t* colind, const
 }  // namespace
 
 using namespace ph;
+
+extern "C" ph_status ph_test_pcg_loop(int mode) {
+  if (mode < 0 || mode > 1) return PH_ERR_ARG;
+  g_test_pcg_loop.store(mode);
+  return PH_OK;
+}
 
 extern "C" ph_status ph_solve_pcg(int64_t n, const int32_t* rowptr, const int32_t* colind, const double* values,
                                   const double* b, double* x, double rtol, int32_t maxit, int32_t* iters,
