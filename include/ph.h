@@ -534,7 +534,9 @@ ph_status ph_kernel_time(const char* kernel, int reset, double* ms, int64_t* lau
  *     affected.  Off by default; for tests only.
  *   ph_test_pcg_loop(mode): 1 makes the conjugate-gradient solves run their
  *     per-iteration kernels where they would run all iterations in one launch
- *     (the same bits); 0 (the default) does not.
+ *     (the same bits); 2 makes one block of that launch never arrive where the
+ *     blocks meet, and all give up after 2^12 polls: the solve returns
+ *     PH_ERR_TIMEOUT; 0 (the default) neither.
  *   ph_pool_in_use(bytes): (host) bytes of the current device's library pool
  *     held by live allocations (freed memory counts once its stream-ordered
  *     free has run), to check that failed calls leak nothing.

@@ -540,7 +540,8 @@ def ph_test_scan_withhold(on):
 
 
 def ph_test_pcg_loop(mode):
-    """Test hook: 1 keeps solves from the one-launch loop, 0 does not."""
+    """Test hook: 1 keeps solves from the one-launch loop, 2 lets a block of it
+    never arrive (the bounded waits run out), 0 neither."""
     _check(load().ph_test_pcg_loop(int(mode)), "ph_test_pcg_loop")
 
 

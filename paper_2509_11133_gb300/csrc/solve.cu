@@ -345,6 +345,7 @@ struct LoopArgs {
   Scalars* sc;
   double tol, res;           // rtol ||b||, the residual norm so far
   int it, it_stop, maxit, spin_limit;
+  int withhold;              // block that never arrives (test hook), or -1
   int rows, slots;           // rows of a slot, slots per block
   SchwarzGroups g;
   int wfirst[kSchwarzDense + 2];  // group k's patches take the warps [wfirst[k], wfirst[k + 1]) of 32
@@ -355,11 +356,12 @@ struct LoopArgs {
 
 // All blocks of the grid meet (they are co-resident: a cooperative launch).
 // Bounded: *late is set, and the call returns, when the wait runs out.
-__device__ __forceinline__ void loop_meet(unsigned* bar, unsigned& target, int spin_limit, int* late) {
+__device__ __forceinline__ void loop_meet(unsigned* bar, unsigned& target, int spin_limit, int withhold, int* late) {
   __syncthreads();
   target += gridDim.x;
   if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    if ((int)blockIdx.x != withhold)
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     unsigned seen;
     for (int spins = 0;; ++spins) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
@@ -587,7 +589,7 @@ __global__ void __launch_bounds__(RT, SCHW ? 2 : 3) k_pcg_loop(const __grid_cons
       }
     }
   }
-  loop_meet(A.bar, target, A.spin_limit, &s_late);
+  loop_meet(A.bar, target, A.spin_limit, A.withhold, &s_late);
 
   while (!s_late && res > A.tol && it < A.maxit && it < A.it_stop) {
     const int batch = min(8, A.maxit - it);
@@ -613,7 +615,7 @@ __global__ void __launch_bounds__(RT, SCHW ? 2 : 3) k_pcg_loop(const __grid_cons
         }
         publish_rows(part_pq, b, v);
       }
-      loop_meet(A.bar, target, A.spin_limit, &s_late);
+      loop_meet(A.bar, target, A.spin_limit, A.withhold, &s_late);
       if (s_late) break;
       const double2 pa = loop_total<WARPS>(part_pq, nscal, [&](double v) { return v > 0.0 ? rz / v : 0.0; });
       pq = pa.x;
@@ -677,7 +679,7 @@ __global__ void __launch_bounds__(RT, SCHW ? 2 : 3) k_pcg_loop(const __grid_cons
         publish_pairs(b, vz, !SCHW, vr, test);
       }
       double2 zb;  // r.z and beta
-      loop_meet(A.bar, target, A.spin_limit, &s_late);
+      loop_meet(A.bar, target, A.spin_limit, A.withhold, &s_late);
       if (s_late) break;
       if (test) {
         rr = loop_total<WARPS>(pair_rr, npair, total_only).x;
@@ -701,7 +703,7 @@ __global__ void __launch_bounds__(RT, SCHW ? 2 : 3) k_pcg_loop(const __grid_cons
           }
           publish_rows(part_rz, b, v);
         }
-        loop_meet(A.bar, target, A.spin_limit, &s_late);
+        loop_meet(A.bar, target, A.spin_limit, A.withhold, &s_late);
         if (s_late) break;
         zb = loop_total<WARPS>(part_rz, nscal, beta_of);
       } else {
@@ -743,7 +745,9 @@ __global__ void __launch_bounds__(RT, SCHW ? 2 : 3) k_pcg_loop(const __grid_cons
 }
 
 constexpr int kLoopSpinLimit = 1 << 21;  // polls (about a microsecond each)
-// Test hook (ph_test_pcg_loop): 1 keeps the solver from k_pcg_loop.
+// Test hook (ph_test_pcg_loop): 1 keeps the solver from k_pcg_loop; 2 lets its first
+// block never arrive, and the polls of all run out after kLoopTestSpinLimit.
+constexpr int kLoopTestSpinLimit = 1 << 12;
 std::atomic<int> g_test_pcg_loop{0};
 constexpr int kLoopIters = 4096;         // iterations per launch (a multiple of 16: the buffers end where they began)
 
@@ -873,7 +877,8 @@ ph_status pcg_run(int64_t n, const int32_t* rowptr, const int32_t* colind, const
     L.it = it;
     L.it_stop = it + kLoopIters;
     L.maxit = maxit;
-    L.spin_limit = kLoopSpinLimit;
+    L.spin_limit = hook == 2 ? kLoopTestSpinLimit : kLoopSpinLimit;
+    L.withhold = hook == 2 ? 0 : -1;
     L.mem = P ? P->mem : nullptr;
     L.fslot = P ? P->fslot : nullptr;
     L.blk = P ? P->blk : nullptr;
@@ -936,7 +941,7 @@ ph_status pcg_run(int64_t n, const int32_t* rowptr, const int32_t* colind, const
 using namespace ph;
 
 extern "C" ph_status ph_test_pcg_loop(int mode) {
-  if (mode < 0 || mode > 1) return PH_ERR_ARG;
+  if (mode < 0 || mode > 2) return PH_ERR_ARG;
   g_test_pcg_loop.store(mode);
   return PH_OK;
 }
