@@ -692,6 +692,10 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_connect(const SmallMesh
   for (int64_t i = tid; i < nE + nN; i += kSmallThreads)
     face_count_item(i, m.tet_in, nE, m.nC, m.nb, nN, m.sub, m.cnt, m.tet, m.status);
   __syncthreads();
+  if (failed(m.status)) {  // invalid ids: nothing may be read through them
+    if (tid == 0) m.d_tot[0] = -1;
+    return;
+  }
   small_scan(m.nbuckets, [&](int64_t i) { return m.cnt[i]; }, m.start);
   for (int64_t i = tid; i < nE + nN; i += kSmallThreads)
     face_fill_item<false>(i, m.tet, nE, m.nC, m.nb, nN, m.sub, m.start, m.cnt, m.entries, m.mate, nullptr, nullptr,
@@ -729,16 +733,18 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_connect(const SmallMesh
                                 m.trel, m.coord, m.face_vtx, m.face_area, none, m.status);
 }
 
-// The geometry of tet i < nE, or the area of face i - nE.
+// The geometry of tet i < nE (also where a face did not match), or the area of
+// face i - nE.
 __global__ void __launch_bounds__(128) k_small_geom(const SmallMesh m) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (failed(m.status)) return;
+  const int64_t nF = m.d_tot[0];
+  if (nF < 0) return;
   if (i < m.nE) {
     tet_geom(m.coord, m.tet[i], i, m.nE >= ph::kFixedMin, m.geo, m.gexp, m.vol, m.status);
     return;
   }
   i -= m.nE;
-  if (i >= m.d_tot[0]) return;
+  if (i >= nF || failed(m.status)) return;
   double p[3][3];
 #pragma unroll
   for (int j = 0; j < 3; ++j)
@@ -1065,7 +1071,12 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
 built:
   free_async(scratch, s);
   scratch = nullptr;
-  if (bits) { st = status_from_bits(bits); goto fail; }
+  if (bits) {
+    // a degenerate tet goes before a face that does not match, also where the
+    // faces are matched first (k_small_connect)
+    st = bits & (1u << PH_ERR_DEGENERATE) ? PH_ERR_DEGENERATE : status_from_bits(bits);
+    goto fail;
+  }
   m->nF = tot[0];
   m->L = tot[1];
   m->nnz = tot[2];
