@@ -505,7 +505,8 @@ ph_status ph_host_mesh_query(const double* coord, int64_t nC, const int32_t* tet
  * Kernel timing, off by default.  `on` is a mask: bit 0 times k_assemble,
  * zero_values (the clearing of values and rhs), k_recover and
  * k_recover_factored; bit 1 the mesh-build kernels
- * (k_face_count, k_face_fill, k_face_match, k_face_emit, k_row_fill) and
+ * (k_face_count, k_face_fill, k_face_match, k_face_emit, k_row_fill; for meshes of
+ * up to 1,536 tets k_small_connect and k_small_geom, which do their work) and
  * the scans (k_scan); 0 switches timing off.  A timed launch
  * is bracketed by a pair of CUDA events on the stream it runs on (not while
  * that stream is being captured into a graph); the events come from a pool

@@ -980,10 +980,16 @@ static ph_status mesh_build(const double* coord, int64_t nC, const int32_t* tet,
                        rowlen, entries, mate, d_tot, m->coord, m->tet, m->tface, m->tmult, m->face_tet, m->face_vtx,
                        m->face_mult, m->rowptr, m->colind, reinterpret_cast<int32_t*>(m->tpos), m->face_kind,
                        reinterpret_cast<unsigned short*>(m->trel), m->geo, m->face_area, m->gexp, m->vol, m->status};
-    k_small_connect<<<1, kSmallThreads, 0, s>>>(sm);
-    PH_CU(launched(), "k_small_connect");
-    k_small_geom<<<grid_for(nE + nFmax, 128), 128, 0, s>>>(sm);
-    PH_CU(launched(), "k_small_geom");
+    {
+      KernelTimer kt("k_small_connect", s, 2);
+      k_small_connect<<<1, kSmallThreads, 0, s>>>(sm);
+      PH_CU(launched(), "k_small_connect");
+    }
+    {
+      KernelTimer kt("k_small_geom", s, 2);
+      k_small_geom<<<grid_for(nE + nFmax, 128), 128, 0, s>>>(sm);
+      PH_CU(launched(), "k_small_geom");
+    }
     PH_TRY(read_counters(d_tot, 3, m->status, s, tot, &bits));
     goto built;
   }

@@ -1,6 +1,6 @@
-"""Meshes with two faults report the same one whether their connectivity is built
-by one block (up to 1,536 tets) or by the general kernels: invalid ids before
-degenerate tets before faces that do not match."""
+"""The two builds of a mesh, by one block (up to 1,536 tets) and by the general
+kernels: a mesh with two faults reports the same one from both (invalid ids
+before degenerate tets before faces that do not match), and both can be timed."""
 import numpy as np
 import pytest
 
@@ -42,3 +42,22 @@ def test_first_fault(m):
     assert code(flat, wrong) == "PH_ERR_ARG"
     assert code(flat, np.vstack([wrong, thrice])) == "PH_ERR_ARG"
     ph.Mesh(cu(coord, torch.float64), cu(tet, torch.int32)).close()
+
+
+@pytest.mark.parametrize("m,kernels", [(6, ("k_small_connect", "k_small_geom")), (7, ("k_face_fill", "k_row_fill"))])
+def test_build_kernels_are_timed(m, kernels):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2509_11133_gb300 as ph
+    ph.load()
+    coord, tet = meshgen.kuhn_cube(m)
+    for k in kernels:
+        ph.ph_kernel_time(k, reset=True)
+    ph.ph_timing_enable(2)
+    try:
+        ph.Mesh(cu(coord, torch.float64), cu(tet, torch.int32)).close()
+    finally:
+        ph.ph_timing_enable(0)
+    for k in kernels:
+        ms, n = ph.ph_kernel_time(k, reset=True)
+        assert n == 1 and ms > 0.0
