@@ -298,14 +298,15 @@ ph_status ph_solve_pcg_noalloc(int64_t n, const int32_t* rowptr, const int32_t* 
  *                     (uD_face, gN_face, factor may be NULL arrays or hold
  *                     NULL entries) and a host array c[n]; uploads a
  *                     descriptor table and synchronises `stream`.
- *   ph_batch_assemble enqueue the two kernels; no allocation, no
+ *   ph_batch_assemble enqueue the two kernels (and the recovery's, if one is
+ *                     bound); no allocation, no
  *                     synchronisation (capturable).
- *   ph_batch_autotune time the candidate configurations (tiles of 256..16384
- *                     elements, 64..256 threads, 2..8 blocks per SM) `reps`
- *                     times each on the bound problems, keep the fastest and
- *                     return its time per batch in *best_ms (host).
+ *   ph_batch_autotune time the present configuration and the candidates (tiles
+ *                     of 256..16384 elements, 64..256 threads, 2..8 blocks per
+ *                     SM) `reps` times each on the bound problems, keep the
+ *                     fastest and return its time per batch in *best_ms (host).
  *   ph_batch_set_config / ph_batch_get_config  the configuration in use.
- *   ph_batch_graph_launch  on first use, capture the two launches into a CUDA
+ *   ph_batch_graph_launch  on first use, capture the launches into a CUDA
  *                     graph (instantiated once; ph_batch_set_config and the
  *                     autotuner reset it, ph_batch_bind keeps it valid since
  *                     it rewrites the descriptor table in place), then launch

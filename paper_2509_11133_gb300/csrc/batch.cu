@@ -7,9 +7,9 @@
 // runs the plain path's per-element code (assemble_element) on the tile's
 // elements, so every problem's values, rhs and factor are bit-identical to a
 // plain ph_assemble call.  Values and rhs are cleared first by one batched zero
-// kernel.  The tile size and block shape come
-// from ph_batch_autotune, which times candidate configurations on the bound
-// problems; the two launches can be instantiated once as a CUDA graph.
+// kernel.  ph_batch_autotune times candidate tile sizes and block shapes on the
+// bound problems; the two launches (three with the recovery) can be instantiated
+// once as a CUDA graph.
 #include <math.h>
 #include <string.h>
 
@@ -348,12 +348,29 @@ extern "C" ph_status ph_batch_autotune(ph_batch* b, int32_t reps, float* best_ms
   cudaStream_t s = (cudaStream_t)stream;
   static const int32_t tiles[] = {256, 1024, 4096, 16384};
   static const int32_t threads[] = {64, 128, 256};
-  static const int32_t bps[] = {2, 4, 8};
+  static const int32_t bps[] = {2, 4, 6, 8};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaError_t e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   float best = 1e30f;
   int32_t bt = b->tile, bth = b->threads, bb = b->blocks_per_sm;
+  const auto time_config = [&] {  // b's present one
+    e = launch_batch(b, s);  // warm-up
+    if (e == cudaSuccess) e = cudaEventRecord(e0, s);
+    for (int32_t r = 0; r < reps && e == cudaSuccess; ++r) e = launch_batch(b, s);
+    if (e == cudaSuccess) e = cudaEventRecord(e1, s);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    float ms = 0.f;
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    ms /= (float)reps;
+    if (e == cudaSuccess && ms < best) {
+      best = ms;
+      bt = b->tile;
+      bth = b->threads;
+      bb = b->blocks_per_sm;
+    }
+  };
+  if (e == cudaSuccess) time_config();  // what the batch runs now, which need not be a candidate
   for (int32_t tl : tiles) {
     if (e != cudaSuccess) break;
     ph_status st = ph_batch_set_config(b, tl, b->threads, b->blocks_per_sm, stream);
@@ -367,20 +384,7 @@ extern "C" ph_status ph_batch_autotune(ph_batch* b, int32_t reps, float* best_ms
         if (e != cudaSuccess) break;
         b->threads = th;
         b->blocks_per_sm = bp;
-        e = launch_batch(b, s);  // warm-up
-        if (e == cudaSuccess) e = cudaEventRecord(e0, s);
-        for (int32_t r = 0; r < reps && e == cudaSuccess; ++r) e = launch_batch(b, s);
-        if (e == cudaSuccess) e = cudaEventRecord(e1, s);
-        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-        float ms = 0.f;
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-        ms /= (float)reps;
-        if (e == cudaSuccess && ms < best) {
-          best = ms;
-          bt = tl;
-          bth = th;
-          bb = bp;
-        }
+        time_config();
       }
   }
   if (e0) cudaEventDestroy(e0);
@@ -395,7 +399,7 @@ extern "C" ph_status ph_batch_graph_launch(ph_batch* b, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
   if (!b->exec) {
-    // capture the two launches on a private stream and instantiate once
+    // capture the launches on a private stream and instantiate once
     cudaStream_t cs = nullptr;
     e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);

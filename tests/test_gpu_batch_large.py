@@ -72,3 +72,24 @@ def test_build_and_kernels():
     b.close()
     for m in together:
         m.close()
+
+
+def test_autotune_times_the_present_configuration():
+    """Every candidate (4 tiles, 3 thread counts, 4 blocks per SM) and the one in
+    use, which need not be among them, are timed: two launches, warm-up and reps."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2509_11133_gb300 as ph
+    ph.load()
+    coord, tet = meshgen.kuhn_cube(4)
+    m = ph.Mesh(cu(coord), cu(tet, torch.int32))
+    new = lambda n: torch.zeros(n, dtype=torch.float64, device="cuda")
+    b = ph.Batch([m])
+    b.bind([cu(np.ones(m.nE))], [1.0], [cu(np.ones(m.nF))], [new(m.nnz)], [new(m.L)])
+    b.set_config(777, 96, 5)
+    before = ph.ph_launch_count()
+    ms = b.autotune(reps=2)
+    assert ph.ph_launch_count() - before == 2 * (1 + 2) * (4 * 3 * 4 + 1)
+    assert ms > 0.0 and b.get_config()["threads"] in (64, 96, 128, 256)
+    b.close()
+    m.close()
