@@ -98,6 +98,11 @@ typedef struct {
  * det = 0; PH_ERR_OVERFLOW when 16 nE + nN or nC reaches 2^31 - 1; a
  * look-back wait of a scan that timed out gives PH_ERR_TIMEOUT.  On error
  * *out is NULL.
+ * Meshes of 32,768 tets and more hold their element geometry in fixed point
+ * (64-bit integers, except for elements whose edges differ by more than a factor of
+ * about 11 or lie outside its exponent range), smaller ones in fp64.  Neither is
+ * less accurate, but the last bits of H, rhs, U and the gradient differ between
+ * the two, and with them an iterative solve within its rtol.
  * Release with ph_mesh_destroy.
  */
 ph_status ph_mesh_create(const double* coord, int64_t nC, const int32_t* tet, int64_t nE,

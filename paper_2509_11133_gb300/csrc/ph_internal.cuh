@@ -137,14 +137,17 @@ inline ph_status status_from_bits(unsigned bits) {
   return PH_OK;
 }
 
-// Meshes of at least so many tets get the fixed-point record (fixed.cuh), smaller
-// ones the fp64 record.  The two differ in the last bits of Q, which an
-// unconverged Jacobi solve (7,000 iterations at 23,328 tets, rtol 1e-10) turns
-// into 4e-9 of Lambda: systems of the size that is solved that way keep their
-// bits.  There the FP64 pipe is not yet the bound: fixed point takes 9.7 us for
-// 11.8 of k_assemble at 16,464 tets, 13.8 for 16.2 at 34,992, 22 for 31 at
-// 95,832, 49 for 82 at 296,352; k_face_fill 8.5 for 8.6, 9.6 for 10.2, 13.5
-// for 15.9, 23 for 31.  The recovery follows the same rule.
+// Meshes of at least so many tets get the fixed-point record (fixed.cuh) and the
+// fixed-point recovery, smaller ones fp64.  This is not where the times cross (fixed
+// point takes 9.7 us for 11.8 of k_assemble at 16,464 tets already, 13.8 for 16.2 at
+// 34,992, 22 for 31 at 95,832, 49 for 82 at 296,352; k_face_fill 8.5 for 8.6, 9.6
+// for 10.2, 13.5 for 15.9, 23 for 31), nor a bound on errors (fixed point has the
+// smaller ones).  Both give H to its last bits, but not the same bits, and a solve
+// that stops at rtol passes such a change on: 4e-9 of Lambda after the 7,000 Jacobi
+// iterations of a 23,328-tet mesh at rtol 1e-10, while both are within rtol.  The
+// line keeps the bits of fp64 for the meshes on which the gain is a few
+// microseconds; above it the last bits of H, rhs, U and the gradient differ from
+// fp64's, and a solve's result by what its rtol allows.
 constexpr int64_t kFixedMin = 32768;
 
 constexpr int kThreads = 256;
