@@ -99,10 +99,10 @@ typedef struct {
  * look-back wait of a scan that timed out gives PH_ERR_TIMEOUT.  On error
  * *out is NULL.
  * Meshes of 32,768 tets and more hold their element geometry in fixed point
- * (64-bit integers, except for elements whose edges differ by more than a factor of
- * about 11 or lie outside its exponent range), smaller ones in fp64.  Neither is
- * less accurate, but the last bits of H, rhs, U and the gradient differ between
- * the two, and with them an iterative solve within its rtol.
+ * (64-bit integers, except for elements with edges or extents too different for
+ * one scale), smaller ones in fp64.  Neither is less accurate, but the last bits
+ * of H, rhs, U and the gradient differ between the two, and with them an iterative
+ * solve within its rtol.
  * Release with ph_mesh_destroy.
  */
 ph_status ph_mesh_create(const double* coord, int64_t nC, const int32_t* tet, int64_t nE,
@@ -250,7 +250,11 @@ ph_status ph_recover_factored_dw(const ph_mesh* mesh, const double* factor, doub
  * workspace (and a copy of H where its rows hold at most 16 entries) from the
  * library's pool and synchronises `stream` every 8 iterations, or for systems
  * of at most 311,296 rows every 4096 (their test runs on the device, in one
- * cooperative launch).  A device-side wait that runs out gives PH_ERR_TIMEOUT.
+ * cooperative launch; x 16-byte aligned).  That launch starts once all its blocks
+ * fit on the device at the same time, so do not make a kernel that holds the
+ * multiprocessors wait for the solve; this goes for ph_solve_pcg_schwarz,
+ * ph_solve_refined and ph_solve_pcg_noalloc too.  A device-side wait that runs out
+ * gives PH_ERR_TIMEOUT.
  * Errors: PH_ERR_NOT_CONVERGED when maxit is reached (x holds the last
  * iterate); PH_ERR_ARG for a non-positive diagonal entry.
  */

@@ -69,7 +69,8 @@ __device__ __forceinline__ void load_problem(ProbDesc& d, const ProbDesc* __rest
 // sits in shared memory and is read again for every element: in registers its
 // 20 fields, with a copy of the element code for each of the eight flag
 // combinations, took 164 of them and left 12 warps on an SM, enough while the
-// FP64 pipe bound the kernel.  MAXT threads at most per block.
+// FP64 pipe bound the kernel.  MAXT threads at most per block; 80 registers with
+// 140 bytes of spill stores for 256, 64 with 320 for 1024.
 template <int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) k_batch_assemble(const ProbDesc* __restrict__ probs,
                                                                const Tile* __restrict__ tiles, int64_t ntiles) {
@@ -205,8 +206,9 @@ extern "C" ph_status ph_batch_create(ph_mesh* const* meshes, int32_t n, void* st
   b->exec = nullptr;
   b->bound = false;
   b->recover = false;
-  // 256 problems, 37.2M tets, assembly and recovery: 9.2 ms; 128 x 4 9.7, 256 x 3
-  // 9.4, 256 x 8 9.6 (more blocks than fit even out the tiles' ends)
+  // 256 problems, 37.2M tets, assembly and recovery: 9.2 ms (8.7 since the recovery
+  // runs in fixed point); 128 x 4 9.7, 256 x 3 9.4, 256 x 8 9.6 (more blocks than fit
+  // even out the tiles' ends)
   b->tile = 1024;
   b->threads = 256;
   b->blocks_per_sm = 6;

@@ -488,9 +488,10 @@ __device__ __forceinline__ int rank7(const int c[7], int x) {
 //    tets (all distinct): 7 candidates with PH_NO_MULT for absent ones, put in
 //    order by a 16-comparator sorting network, all in registers.  The thread
 //    also computes the face's area, whose 22 FP64 operations bound the kernel
-//    (1.49 ms at 35.9M faces; with the product in fixed point 1.35, but see
-//    fixed.cuh on the areas' last bits).  All loads are issued before the
-//    first use, so the other chains of gathers hide under the FP64 pipe.
+//    (1.50 ms at 35.9M faces; with the product in fixed point 1.35, but see
+//    fixed.cuh on the areas' last bits).  Its chains of gathers hide under the
+//    FP64 pipe in any order: issuing all loads first changed nothing (1.49 ms
+//    before).
 // BATCH (a batched build): U holds the problems' offsets; the face's ids (in
 // place), its column ids and positions are then local to its problem.
 struct FillOffsets {
@@ -510,8 +511,7 @@ __device__ __forceinline__ void row_fill_item(int64_t F, int2* __restrict__ face
                            int32_t* __restrict__ face_vtx, double* __restrict__ area, const FillOffsets U,
                            unsigned* status) {
   if (F >= nFmax || F >= d_tot[0] || failed(status)) return;
-  // every load whose address is known, before anything uses one: the vertices'
-  // and the tets' chains of loads run side by side
+  // every load whose address is known, before anything uses one
   const int2 ft = face_tet[F];
   const int l = face_mult[F];
   const int T[2] = {ft.x, ft.y};
