@@ -14,8 +14,8 @@
 // integer: sum of v w = 2^64 sum(h h') + 2^32 sum(h l' + l h') + sum(l l'),
 // and the last sum, below 2^62 per term, is left out where the result keeps no bits
 // below it, and kept (mac_wide) where the sum is shifted further: left out of Y
-// (a shift of 6) it cost Q up to 10.7 x 2^-53 of its largest entry, now 4.2 at worst
-// and 1.4 rms at most over the shapes that are accepted; fp64: 17 and 3.4.
+// (a shift of 6) it cost Q up to 10.7 x 2^-53 of its largest entry, now 4.4 at worst
+// and 1.2 rms at most over the shapes that are accepted; fp64: 22 and 3.4.
 // Sums of at most three products do not overflow with |v|, |w| <= 2^61:
 // |h l'| <= 2^60, six of them 2^62.6.  The high sum may be shifted past 2^63 on
 // the way (two's complement): only the final value has to fit.
@@ -121,7 +121,7 @@ FX_HD double to_double(int64_t v, int k) {
 // infinity among them).  So every entry is as accurate as in fp64, over regular,
 // jittered, flat, needle and short-edged elements against binary128: diagonal
 // entries to 0.6 x 2^-53 (rms; 0.7 at most for a shape) where fp64 has 0.8, 1.5
-// against 2.8 at worst, and with them the contraction with adj(G) of the gradient
+// against 2.9 at worst, and with them the contraction with adj(G) of the gradient
 // (median, 90th and 99th percentile of the error 0.7 to 1.0 of fp64's).
 // |det E| and the face areas stay fp64: they carry the leading term d d'/(c|T|) of
 // H, whose last bit an ill-conditioned solve amplifies by 1e7, and rounding them
